@@ -117,8 +117,8 @@ typedef struct {
   int32_t threads_per_cta; /* batched mode: threads per scenario CTA; 0 = tuned/default */
   int32_t ctas_per_sm;     /* batched mode: resident CTAs per SM; 0 = tuned/default */
   int32_t kernel_variant;  /* batched mode: register-budget variant 0..2 of the persistent kernel
-                              (0: no cap, small active-set rounds on lane groups; 1: 32 threads x
-                              12 CTAs/SM; 2: 64 threads x 8 CTAs/SM); results are the same bits */
+                              (0: no cap; 1: 32 threads x 12 CTAs/SM; 2: 64 threads x 8 CTAs/SM);
+                              results are the same bits */
   int32_t flags;           /* TADMM_FLAG_* bits; 0 = all optimizations on */
   /* Residual balancing of the penalty (an extension: the paper keeps rho fixed;
    * Boyd et al. 2011, Sec. 3.4.1).  Every adapt_every iterations (0 = off), after
@@ -146,7 +146,7 @@ typedef struct {
                                              FP32 pipe instead of the FP64 pipe; results agree with
                                              float64 to about 1e-13 relative */
 #define TADMM_FLAG_NO_LANE_GROUPS 16      /* stage refactorizations and EQP passes one lane per agent, never
-                                             spread over a group of lanes (bitwise the same results) */
+                                             one lane per axis of an agent (bitwise the same results) */
 #define TADMM_FLAG_NO_COOP_REFACTOR TADMM_FLAG_NO_LANE_GROUPS
 
 typedef struct tadmm_handle tadmm_handle;

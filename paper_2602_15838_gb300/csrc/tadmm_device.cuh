@@ -5,9 +5,9 @@
 // kernels of the plain and graph modes share them:
 //   x-update  (K-a)  one lane per agent, all lanes of a warp together:
 //                    Riccati-factorized primal active set for the
-//                    box-constrained local QP (Sec. IV.A-C); stage
-//                    refactorizations (and, in the per-phase kernels, EQP
-//                    passes) spread over lane groups when few agents need them;
+//                    box-constrained local QP (Sec. IV.A-C); for the double
+//                    integrator in tadmm_axis.cuh, one lane per axis of an
+//                    agent when few agents need a solve;
 //   pair      (K-b)  per (pair, step): halfspace projection of the consensus
 //                    copies, scaled dual update and residuals;
 //   gather    (K-b') per (agent, step): the aggregate linear term of the next
@@ -19,8 +19,9 @@
 //   h       [T][DP][N]     sum over partners of (w - y), t = 1..T
 //   U, Us   [T][NU][N]     current active-set iterate and EQP solution
 //   Wm, Cm  [T][N]         working-set and cached-factor bit masks
-//   cache   [T+1][E][N]    Riccati cache per stage (CacheLayout): P_t, K_t,
-//                          S_t^{-1}, k_t, P_{t+1}B, B'p_{t+1}
+//   cache   [T+1][E][N]    Riccati cache per stage: P_t, K_t, S_t^{-1}, k_t,
+//                          P_{t+1}B, B'p_{t+1} (CacheLayout; AxisCache for the
+//                          double integrator, [T+1][word][axis][N])
 //   theta   [slot][T][P]   projection steps theta^k (multiplier / rho), three
 //                          slots rotating with k mod 3
 //   a       [T][DP][P]     halfspace normals
@@ -90,7 +91,7 @@ struct Dev {
   int32_t as_max;            // 0: 10*T*NU + 10
   double eps_rel;
   int32_t single_as_group;   // 1: a lone scenario of at most 32 agents also runs the group path
-  int32_t coop;              // 1: refactorizations may be spread over lane groups
+  int32_t coop;              // 1: few agents' solves may take one lane per axis
   int32_t adapt_every;       // residual balancing of rho every adapt_every iterations (0: off)
   double adapt_mu, adapt_tau;
   int32_t relax;             // 1: over-relaxed consensus/dual update with factor alpha (group path)
@@ -273,7 +274,7 @@ struct AgentCtx {
   const F* qf;       // the agent's rows of Qf, x_ref and x_init
   const F* xr;
   const F* xi;
-  int coop;          // cooperative refactorization allowed (uniform over the warp)
+  int coop;          // one lane per axis allowed (uniform over the warp)
   int nc;            // consensus copies of the agent (its number of pairs)
 
   __device__ __forceinline__ F k(int e) const { return kc[e * ks]; }
@@ -472,45 +473,24 @@ __device__ __forceinline__ int factor_stage(const Model<F, NX, NU>& Mo, const F 
 
 // ---------------------------------------------------------------------------
 // Stage factorizations of a warp's agents (the refactorization part of the
-// Riccati backward recursion, Sec. IV.B), taken before an EQP pass.  Every
-// lane of the warp calls this together; `own` marks the lanes whose agent
-// needs stages dirty..0 refactored.  When few agents need it, the work of each
-// agent's stage is spread over a group of lanes (one lane per row of P): the
-// FP64 pipe costs the warp the same per instruction whatever the number of
-// active lanes, so a refactorization that serves a handful of agents is
-// otherwise paid at full price.  Each value is formed by the same operations,
-// in the same order, as in factor_stage, so both forms give identical bits.
+// Riccati backward recursion, Sec. IV.B), taken before an EQP pass: one lane
+// per agent, dense products.  Every lane of the warp calls this together; `own`
+// marks the lanes whose agent needs stages dirty..0 refactored.
 // ---------------------------------------------------------------------------
-template <int NX>
-struct CoopShape {
-  static constexpr int GS = NX <= 4 ? 4 : 8;      // lanes per agent group
-  static constexpr int NG = 32 / GS;               // groups per warp
-  static constexpr int MAXOWN = NX <= 4 ? 16 : 16; // largest owner count taken cooperatively
-};
-
 template <typename F>
 __device__ __forceinline__ F shfl_f(F v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-
-// v[idx] for a lane-dependent idx without local-memory indexing.
-template <typename F, int N>
-__device__ __forceinline__ F pick(const F (&v)[N], int idx) {
-  F r = v[0];
-#pragma unroll
-  for (int c = 1; c < N; ++c)
-    if (idx == c) r = v[c];
-  return r;
+__device__ __forceinline__ df64 shfl_f(df64 v, int src) {
+  return df64(__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src));
 }
 
-template <typename F, int NX, int NU, int DP, bool DI>
+template <typename F, int NX, int NU, int DP>
 __device__ void refactor_sweep(const AgentCtx<F, NX, NU, DP>& A, bool own, int dirty, unsigned long long& nfact,
                                int& bad_out) {
   using CL = CacheLayout<NX, NU>;
   using AC = AgentConst<NX, NU>;
   constexpr unsigned FULL = 0xffffffffu;
-  const unsigned owners = __ballot_sync(FULL, own && dirty >= 0);
-  if (!owners) return;
-  const int lane = threadIdx.x & 31;
   const bool mine = own && dirty >= 0;
+  if (!__any_sync(FULL, mine)) return;
   if (mine && dirty >= A.T - 1) {
     // P_T = Qbar_T
 #pragma unroll
@@ -519,188 +499,34 @@ __device__ void refactor_sweep(const AgentCtx<F, NX, NU, DP>& A, bool own, int d
       for (int c = 0; c < NX; ++c) A.C(A.T, CL::P + r * NX + c) = (r == c) ? A.qbarT(r) : F(0);
   }
   if (mine) nfact += (unsigned long long)(dirty + 1);
+  const int maxd = __reduce_max_sync(FULL, mine ? dirty : -1);
   __syncwarp();
-  const int n = __popc(owners);
-  constexpr bool coop_type = std::is_same<F, double>::value || std::is_same<F, float>::value;
-  if (!(DI && coop_type) || n > CoopShape<NX>::MAXOWN || !A.coop) {
-    // one lane per agent
-    const int maxd = __reduce_max_sync(FULL, mine ? dirty : -1);
-    __syncwarp();
-    for (int t = maxd; t >= 0; --t) {
-      if (mine && t <= dirty) {
-        const uint16_t mask = A.W(t);
-        F Pn[NX][NX], K[NU][NX], L[NU][NU];
+  for (int t = maxd; t >= 0; --t) {
+    if (mine && t <= dirty) {
+      const uint16_t mask = A.W(t);
+      F Pn[NX][NX], K[NU][NX], L[NU][NU];
 #pragma unroll
-        for (int r = 0; r < NX; ++r)
+      for (int r = 0; r < NX; ++r)
 #pragma unroll
-          for (int c = 0; c < NX; ++c) Pn[r][c] = A.C(t + 1, CL::P + r * NX + c);
-        auto put = [&](int r, int c, F v) {
-          A.C(t, CL::P + r * NX + c) = v;
-          if (c != r) A.C(t, CL::P + c * NX + r) = v;
-        };
-        auto putB = [&](int r, int a, F v) { A.C(t, CL::PB + r * NU + a) = v; };
-        bad_out |= factor_stage<F, NX, NU, DI>(*A.M, Pn, mask, A.kc + AC::RB * A.ks,
-                                               t >= 1 ? A.kc + AC::QB * A.ks : nullptr, A.ks, put, putB, K, L);
+        for (int c = 0; c < NX; ++c) Pn[r][c] = A.C(t + 1, CL::P + r * NX + c);
+      auto put = [&](int r, int c, F v) {
+        A.C(t, CL::P + r * NX + c) = v;
+        if (c != r) A.C(t, CL::P + c * NX + r) = v;
+      };
+      auto putB = [&](int r, int a, F v) { A.C(t, CL::PB + r * NU + a) = v; };
+      bad_out |= factor_stage<F, NX, NU, false>(*A.M, Pn, mask, A.kc + AC::RB * A.ks,
+                                                t >= 1 ? A.kc + AC::QB * A.ks : nullptr, A.ks, put, putB, K, L);
 #pragma unroll
-        for (int a = 0; a < NU; ++a) {
+      for (int a = 0; a < NU; ++a) {
 #pragma unroll
-          for (int c = 0; c < NX; ++c) A.C(t, CL::K + a * NX + c) = K[a][c];
+        for (int c = 0; c < NX; ++c) A.C(t, CL::K + a * NX + c) = K[a][c];
 #pragma unroll
-          for (int b = 0; b <= a; ++b) A.C(t, CL::L + a * NU + b) = L[a][b];
-        }
-        A.CM(t) = mask;
+        for (int b = 0; b <= a; ++b) A.C(t, CL::L + a * NU + b) = L[a][b];
       }
-    }
-    __syncwarp();
-    return;
-  }
-  if constexpr (DI && coop_type) {
-    constexpr int GS = CoopShape<NX>::GS, NG = CoopShape<NX>::NG, H = NX / 2;
-    static_assert(NU == H, "double integrator: one input per position axis");
-    const Model<F, NX, NU>& Mo = *A.M;
-    const F dt = Mo.A[0][H], b1 = Mo.B[0][0], b2 = Mo.B[H][0];
-    const int g = lane / GS, r = lane % GS, gbase = g * GS;
-    const int rr = r < NX ? r : NX - 1;  // row of this lane (lanes past NX mirror the last row, never store)
-    int gbad = 0;
-    unsigned rem = owners;
-    while (rem) {
-      // the next NG owners, in lane order; group g takes the g-th of them
-      unsigned chunk = 0, m = rem;
-      for (int k = 0; k < NG && m; ++k) {
-        chunk |= m & (0u - m);
-        m &= m - 1;
-      }
-      rem &= ~chunk;
-      int olane = -1;
-      {
-        unsigned c2 = chunk;
-        for (int k = 0; k < g && c2; ++k) c2 &= c2 - 1;
-        if (c2) olane = __ffs(c2) - 1;
-      }
-      const int src = olane >= 0 ? olane : lane;
-      F* const ocache = (F*)__shfl_sync(FULL, (unsigned long long)A.cache, src);
-      uint16_t* const oW = (uint16_t*)__shfl_sync(FULL, (unsigned long long)A.Wm, src);
-      uint16_t* const oC = (uint16_t*)__shfl_sync(FULL, (unsigned long long)A.Cm, src);
-      const F* const okc = (const F*)__shfl_sync(FULL, (unsigned long long)A.kc, src);
-      const int oks = __shfl_sync(FULL, A.ks, src);
-      const int oN = __shfl_sync(FULL, A.N, src);
-      const int oi = __shfl_sync(FULL, A.i, src);
-      const int od = __shfl_sync(FULL, mine ? dirty : -1, src);
-      const bool gact = olane >= 0;
-      const int maxd = __reduce_max_sync(FULL, gact ? od : -1);
-      auto OC = [&](int t, int e) -> F& { return ocache[((size_t)t * CL::E + e) * oN + oi]; };
-      for (int t = maxd; t >= 0; --t) {
-        const bool act = gact && t <= od;
-        const bool row = act && r < NX;
-        const uint16_t mask = act ? oW[(size_t)t * oN + oi] : (uint16_t)0;
-        F Pr[NX];
-#pragma unroll
-        for (int c = 0; c < NX; ++c) Pr[c] = act ? OC(t + 1, CL::P + rr * NX + c) : F(0);
-        F PAr[NX], PBr[NU];
-#pragma unroll
-        for (int c = 0; c < H; ++c) {
-          PAr[c] = Pr[c];
-          PAr[H + c] = fma(Pr[H + c], F(1), Pr[c] * dt);
-          PBr[c] = fma(Pr[H + c], b2, Pr[c] * b1);
-        }
-        // rows H + a of PA and PB for the lanes a < NU
-        const int shi = gbase + (r < NU ? r + H : rr);
-        F PAh[NX], PBh[NU];
-#pragma unroll
-        for (int c = 0; c < NX; ++c) PAh[c] = shfl_f(PAr[c], shi);
-#pragma unroll
-        for (int c = 0; c < NU; ++c) PBh[c] = shfl_f(PBr[c], shi);
-        // row ra = min(r, NU - 1) of S and of M = B'P A (fixed rows/cols replaced)
-        const int ra = r < NU ? r : NU - 1;
-        const bool fa = (mask >> ra) & 0x101;
-        F Srow[NU], Mrow[NX];
-#pragma unroll
-        for (int b = 0; b < NU; ++b) {
-          const bool fb = (mask >> b) & 0x101;
-          F acc = (ra == b) ? (act ? okc[(AC::RB + ra) * oks] : F(1)) : F(0);
-          acc = fma(b1, PBr[b], acc);
-          acc = fma(b2, PBh[b], acc);
-          Srow[b] = (fa || fb) ? F(ra == b ? 1 : 0) : acc;
-        }
-#pragma unroll
-        for (int c = 0; c < NX; ++c) {
-          F acc = 0;
-          acc = fma(b1, PAr[c], acc);
-          acc = fma(b2, PAh[c], acc);
-          Mrow[c] = fa ? F(0) : acc;
-        }
-        // S, M on every lane of the group; S^{-1}; column rr of K
-        F S[NU][NU], Mm[NU][NX], Si[NU][NU];
-#pragma unroll
-        for (int a = 0; a < NU; ++a) {
-#pragma unroll
-          for (int b = 0; b < NU; ++b) S[a][b] = shfl_f(Srow[b], gbase + a);
-#pragma unroll
-          for (int c = 0; c < NX; ++c) Mm[a][c] = shfl_f(Mrow[c], gbase + a);
-        }
-        const int sbad = sym_inverse<F, NU>(S, Si);
-        if (act && r == 0) gbad |= sbad;
-        F kcol[NU];
-        {
-          F mc[NU];
-#pragma unroll
-          for (int b = 0; b < NU; ++b) mc[b] = pick<F, NX>(Mm[b], rr);
-          neg_sinv<F, NU>(Si, mc, kcol);
-        }
-        if (row) {
-#pragma unroll
-          for (int a = 0; a < NU; ++a) OC(t, CL::K + a * NX + rr) = kcol[a];
-#pragma unroll
-          for (int a = 0; a < NU; ++a) OC(t, CL::PB + rr * NU + a) = PBr[a];
-        }
-        if (act && r == 0) {
-#pragma unroll
-          for (int a = 0; a < NU; ++a)
-#pragma unroll
-            for (int b = 0; b <= a; ++b) OC(t, CL::L + a * NU + b) = Si[a][b];
-          oC[(size_t)t * oN + oi] = mask;
-        }
-        if (t >= 1) {
-          // P_t row rr: Qbar_t + A'(P A) + M'K, entries c >= rr
-          F K[NU][NX], PAl[NX];
-#pragma unroll
-          for (int c = 0; c < NX; ++c)
-#pragma unroll
-            for (int a = 0; a < NU; ++a) K[a][c] = shfl_f(kcol[a], gbase + c);
-          const int slo = gbase + (rr >= H ? rr - H : rr);
-#pragma unroll
-          for (int c = 0; c < NX; ++c) PAl[c] = shfl_f(PAr[c], slo);
-          const F qd = act ? okc[(AC::QB + rr) * oks] : F(0);
-          F mr[NU];
-#pragma unroll
-          for (int k = 0; k < NU; ++k) mr[k] = pick<F, NX>(Mm[k], rr);
-#pragma unroll
-          for (int c = 0; c < NX; ++c) {
-            if (c < rr) continue;
-            F acc = (rr == c) ? qd : F(0);
-            if (rr < H) {
-              acc = acc + PAr[c];
-            } else {
-              acc = fma(dt, PAl[c], acc);
-              acc = acc + PAr[c];
-            }
-#pragma unroll
-            for (int k = 0; k < NU; ++k) acc = fma(mr[k], K[k][c], acc);
-            if (row) {
-              OC(t, CL::P + rr * NX + c) = acc;
-              if (c != rr) OC(t, CL::P + c * NX + rr) = acc;
-            }
-          }
-        }
-        __syncwarp();
-      }
-      // each owner of the chunk takes its group's status
-      const int gi = __popc(chunk & ((1u << lane) - 1u));
-      const int b = __shfl_sync(FULL, gbad, (mine && ((chunk >> lane) & 1u) ? gi : 0) * GS);
-      if (mine && ((chunk >> lane) & 1u)) bad_out |= b;
-      gbad = 0;
+      A.CM(t) = mask;
     }
   }
+  __syncwarp();
 }
 
 // One EQP solve with the cached stage factors (refactor_sweep brings them up to
@@ -710,9 +536,8 @@ __device__ void refactor_sweep(const AgentCtx<F, NX, NU, DP>& A, bool own, int d
 // P_{t+1} x_{t+1} + p_{t+1} (Sec. IV.B dual recovery), evaluated only at stages
 // that hold fixed inputs, and flags free inputs that left the box (integer
 // keys); the exact ratio test runs only when such an input exists.
-template <typename F, int NX, int NU, int DP, bool DI>
+template <typename F, int NX, int NU, int DP>
 __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
-  constexpr int H = NX / 2;
   using CL = CacheLayout<NX, NU>;
   const Model<F, NX, NU>& Mo = *A.M;
   const int T = A.T;
@@ -776,13 +601,8 @@ __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
 #pragma unroll
       for (int a = 0; a < NU; ++a) {
         F acc = 0;
-        if constexpr (DI) {
-          acc = fma(Mo.B[0][0], pn[a], acc);
-          acc = fma(Mo.B[H][0], pn[H + a], acc);
-        } else {
 #pragma unroll
-          for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], pn[r], acc);
-        }
+        for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], pn[r], acc);
         A.C(t, CL::bp + a) = acc;
       }
     }
@@ -790,13 +610,8 @@ __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
 #pragma unroll
     for (int a = 0; a < NU; ++a) {
       F acc = 0;
-      if constexpr (DI) {
-        acc = fma(Mo.B[0][0], Pcp[a], acc);
-        acc = fma(Mo.B[H][0], Pcp[H + a], acc);
-      } else {
 #pragma unroll
-        for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], Pcp[r], acc);
-      }
+      for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], Pcp[r], acc);
       sv[a] = (mask & (0x101u << a)) ? F(0) : acc;
     }
     neg_sinv<F, NU>(L, sv, kk);
@@ -806,17 +621,8 @@ __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
 #pragma unroll
       for (int r = 0; r < NX; ++r) {
         F acc = A.q_h(r, r < DP ? ht[r] : F(0));
-        if constexpr (DI) {
-          if (r < H) {
-            acc = acc + Pcp[r];
-          } else {
-            acc = fma(Mo.A[0][H], Pcp[r - H], acc);
-            acc = acc + Pcp[r];
-          }
-        } else {
 #pragma unroll
-          for (int k = 0; k < NX; ++k) acc = fma(Mo.A[k][r], Pcp[k], acc);
-        }
+        for (int k = 0; k < NX; ++k) acc = fma(Mo.A[k][r], Pcp[k], acc);
 #pragma unroll
         for (int k = 0; k < NU; ++k) acc = fma(K[k][r], sv[k], acc);
         pn[r] = acc;
@@ -879,22 +685,14 @@ __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
       }
     }
     F xn[NX];
-    if constexpr (DI) {
 #pragma unroll
-      for (int c = 0; c < H; ++c) {
-        xn[c] = fma(Mo.B[0][0], uv[c], fma(Mo.A[0][H], xv[H + c], xv[c]));
-        xn[H + c] = fma(Mo.B[H][0], uv[c], xv[H + c]);
-      }
-    } else {
+    for (int r = 0; r < NX; ++r) {
+      F acc = 0;
 #pragma unroll
-      for (int r = 0; r < NX; ++r) {
-        F acc = 0;
+      for (int c = 0; c < NX; ++c) acc = fma(Mo.A[r][c], xv[c], acc);
 #pragma unroll
-        for (int c = 0; c < NX; ++c) acc = fma(Mo.A[r][c], xv[c], acc);
-#pragma unroll
-        for (int c = 0; c < NU; ++c) acc = fma(Mo.B[r][c], uv[c], acc);
-        xn[r] = acc;
-      }
+      for (int c = 0; c < NU; ++c) acc = fma(Mo.B[r][c], uv[c], acc);
+      xn[r] = acc;
     }
     if (mask) {
 #pragma unroll
@@ -927,248 +725,11 @@ __device__ EqpScan<F> eqp_solve(const AgentCtx<F, NX, NU, DP>& A) {
   return o;
 }
 
-// EQP solve of the agents of up to CoopShape<NX>::NG lanes of the warp, each
-// agent on a group of lanes with one lane per state row: the backward affine
-// pass and the forward rollout exchange rows by warp shuffles, so that an
-// agent's stage recurrence is a few operations long instead of a few dozen.
-// Every value is formed by the same operations, in the same order, as in
-// eqp_solve, so both give identical bits.  Every lane of the warp calls this;
-// `go` marks the lanes whose agent takes the pass (at most NG of them, the
-// caller checks).  The owner lane receives its agent's scan.  Used by the
-// per-phase x-update kernels, where few agents share a warp and each agent's
-// recurrence latency sets the time, and by the register-unbounded variant 0 of
-// the persistent kernel for its later active-set rounds, which serve a few
-// agents of the warp (variant 1's 168-register budget leaves it out).
-template <typename F, int NX, int NU, int DP>
-__device__ EqpScan<F> eqp_coop(const AgentCtx<F, NX, NU, DP>& A, bool go) {
-  constexpr unsigned FULL = 0xffffffffu;
-  constexpr int GS = CoopShape<NX>::GS, H = NX / 2;
-  using CL = CacheLayout<NX, NU>;
-  using AC = AgentConst<NX, NU>;
-  const Model<F, NX, NU>& Mo = *A.M;
-  const F dt = Mo.A[0][H], b1 = Mo.B[0][0], b2 = Mo.B[H][0];
-  const int lane = threadIdx.x & 31, g = lane / GS, r = lane % GS, gbase = g * GS;
-  const int rr = r < NX ? r : NX - 1;  // state row of this lane
-  const int ra = r < NU ? r : NU - 1;  // input of this lane
-  const unsigned owners = __ballot_sync(FULL, go);
-  int olane = -1;
-  {
-    unsigned m = owners;
-    for (int k = 0; k < g && m; ++k) m &= m - 1;
-    if (m) olane = __ffs(m) - 1;
-  }
-  const int src = olane >= 0 ? olane : lane;
-  auto sp = [&](auto p) { return (decltype(p))__shfl_sync(FULL, (unsigned long long)p, src); };
-  F* const cache = sp(A.cache);
-  uint16_t* const Wm = sp(A.Wm);
-  F* const Us = sp(A.Us);
-  F* const Xo = sp(A.Xo);
-  const F* const hp = sp(A.h);
-  const F* const kc = sp(A.kc);
-  const F* const qf = sp(A.qf);
-  const F* const xr = sp(A.xr);
-  const F* const xi = sp(A.xi);
-  const int ks = __shfl_sync(FULL, A.ks, src), N = __shfl_sync(FULL, A.N, src);
-  const int ai = __shfl_sync(FULL, A.i, src), T = __shfl_sync(FULL, A.T, src);
-  const bool gact = olane >= 0;
-  const bool row = gact && r < NX;
-  const int Tm = __reduce_max_sync(FULL, gact ? T : 0);
-  auto C = [&](int t, int e) -> F& { return cache[((size_t)t * CL::E + e) * N + ai]; };
-  const F rho = gact ? kc[AC::RHO * ks] : F(0);
+}  // namespace tadmm
 
-  // backward affine pass; this lane carries p_{t+1}[rr]
-  F pn = F(0);
-  if (gact) {
-    pn = terminal_lin(qf[rr], xr[rr]);
-    if (rr < DP) pn = lin_term(pn, rho, hp[((size_t)(T - 1) * DP + rr) * N + ai]);
-  }
-  // this lane's operands of a stage, loaded one stage ahead: mask, row rr of
-  // P_{t+1}B, row ra of S^{-1}, column rr of K, h_t[rr]
-  uint16_t mk_n = 0;
-  F pb_n[NU], si_n[NU], kq_n[NU], h_n = F(0);
-  auto load_back = [&](int t) {
-    const bool act = gact && t >= 0 && t < T;
-    mk_n = act ? Wm[(size_t)t * N + ai] : (uint16_t)0;
-#pragma unroll
-    for (int a = 0; a < NU; ++a) {
-      pb_n[a] = act ? C(t, CL::PB + rr * NU + a) : F(0);
-      si_n[a] = act ? C(t, CL::L + (a <= ra ? ra * NU + a : a * NU + ra)) : F(0);
-      kq_n[a] = act ? C(t, CL::K + a * NX + rr) : F(0);
-    }
-    h_n = (act && t >= 1 && rr < DP) ? hp[((size_t)(t - 1) * DP + rr) * N + ai] : F(0);
-  };
-  load_back(Tm - 1);
-  for (int t = Tm - 1; t >= 0; --t) {
-    const bool act = gact && t < T;
-    const uint16_t mask = mk_n;
-    F pbv[NU], si[NU], kq[NU];
-#pragma unroll
-    for (int a = 0; a < NU; ++a) {
-      pbv[a] = pb_n[a];
-      si[a] = si_n[a];
-      kq[a] = kq_n[a];
-    }
-    const F hv = h_n;
-    if (t >= 1) load_back(t - 1);
-    F Pcp = pn;
-    if (mask) {
-#pragma unroll
-      for (int a = 0; a < NU; ++a) {
-        if (!(mask & (0x101u << a))) continue;
-        const F ub = (mask & (1u << a)) ? Mo.umin[a] : Mo.umax[a];
-        Pcp = fma(pbv[a], ub, Pcp);
-      }
-    }
-    // rows H + ra of p_{t+1} and of P_{t+1} c + p_{t+1}
-    const int shi = gbase + H + ra;
-    const F pnh = shfl_f(pn, shi), Pcph = shfl_f(Pcp, shi);
-    if (mask && r < NU) {
-      F acc = 0;
-      acc = fma(b1, pn, acc);
-      acc = fma(b2, pnh, acc);
-      C(t, CL::bp + ra) = acc;
-    }
-    F svl = 0;
-    {
-      F acc = 0;
-      acc = fma(b1, Pcp, acc);
-      acc = fma(b2, Pcph, acc);
-      svl = (mask & (0x101u << ra)) ? F(0) : acc;
-    }
-    F sv[NU];
-#pragma unroll
-    for (int b = 0; b < NU; ++b) sv[b] = shfl_f(svl, gbase + b);
-    if (act && r < NU) {
-      // k_t row ra = -(S^{-1} s)[ra]
-      F acc = si[0] * sv[0];
-#pragma unroll
-      for (int b = 1; b < NU; ++b) acc = fma(si[b], sv[b], acc);
-      C(t, CL::k + ra) = -acc;
-    }
-    if (t >= 1) {
-      const F Pcpl = shfl_f(Pcp, gbase + (rr >= H ? rr - H : rr));
-      if (act) {
-        F acc = kc[(AC::QL + rr) * ks];
-        if (rr < DP) acc = lin_term(acc, rho, hv);
-        if (rr < H) {
-          acc = acc + Pcp;
-        } else {
-          acc = fma(dt, Pcpl, acc);
-          acc = acc + Pcp;
-        }
-#pragma unroll
-        for (int k = 0; k < NU; ++k) acc = fma(kq[k], sv[k], acc);
-        pn = acc;
-      }
-    }
-  }
-  __syncwarp();
+#include "tadmm_axis.cuh"
 
-  // forward rollout; this lane carries x_t[rr]
-  EqpScan<F> o;
-  o.anum = 1; o.aden = 1; o.blk = -1; o.bside = 0; o.worst = 0; o.widx = -1; o.scale = 1; o.bad = 0; o.out = 0;
-  const unsigned long long kmin = mono_key(Mo.umin[ra]), kmax = mono_key(Mo.umax[ra]);
-  F xl = gact ? xi[rr] : F(0);
-  if (row) Xo[(size_t)rr * N + ai] = xl;
-  // this lane's operands of a stage, loaded one stage ahead: mask, k_t[ra],
-  // row ra of K_t, B'p_{t+1}[ra], column ra of P_{t+1}B
-  uint16_t fm_n = 0;
-  F kf_n = F(0), Kr_n[NX], bp_n = F(0), pbc_n[NX];
-  auto load_fwd = [&](int t) {
-    const bool act = gact && t < T;
-    fm_n = act ? Wm[(size_t)t * N + ai] : (uint16_t)0;
-    kf_n = act ? C(t, CL::k + ra) : F(0);
-    bp_n = act ? C(t, CL::bp + ra) : F(0);
-#pragma unroll
-    for (int c = 0; c < NX; ++c) {
-      Kr_n[c] = act ? C(t, CL::K + ra * NX + c) : F(0);
-      pbc_n[c] = act ? C(t, CL::PB + c * NU + ra) : F(0);
-    }
-  };
-  load_fwd(0);
-  for (int t = 0; t < Tm; ++t) {
-    const bool act = gact && t < T;
-    const uint16_t mask = fm_n;
-    const F kfv = kf_n, bpv = bp_n;
-    F Kr[NX], pbc[NX];
-#pragma unroll
-    for (int c = 0; c < NX; ++c) {
-      Kr[c] = Kr_n[c];
-      pbc[c] = pbc_n[c];
-    }
-    if (t + 1 < Tm) load_fwd(t + 1);
-    F xv[NX];
-#pragma unroll
-    for (int c = 0; c < NX; ++c) xv[c] = shfl_f(xl, gbase + c);
-    F ul;
-    if (mask & (1u << ra)) ul = Mo.umin[ra];
-    else if (mask & (0x100u << ra)) ul = Mo.umax[ra];
-    else {
-      F acc = kfv;
-#pragma unroll
-      for (int c = 0; c < NX; ++c) acc = fma(Kr[c], xv[c], acc);
-      ul = acc;
-      const unsigned long long ku = mono_key(acc);
-      if (act && r < NU) o.out |= (ku < kmin) | (ku > kmax);
-    }
-    F uv[NU];
-#pragma unroll
-    for (int b = 0; b < NU; ++b) uv[b] = shfl_f(ul, gbase + b);
-    F xn;
-    if (rr < H) xn = fma(b1, pick<F, NU>(uv, rr), fma(dt, pick<F, NX>(xv, H + rr), xl));
-    else xn = fma(b2, pick<F, NU>(uv, rr - H), xl);
-    // every lane takes part in the shuffles (the masks differ between groups)
-    F xnv[NX];
-#pragma unroll
-    for (int c = 0; c < NX; ++c) xnv[c] = shfl_f(xn, gbase + c);
-    if (mask) {
-      if (act && r < NU && (mask & (0x101u << ra))) {
-        F gg = bpv;
-#pragma unroll
-        for (int c = 0; c < NX; ++c) gg = fma(pbc[c], xnv[c], gg);
-        gg = fma(kc[(AC::RB + ra) * ks], ul, gg);
-        const F mu = (mask & (1u << ra)) ? gg : -gg;
-        const unsigned long long ab = abs_bits(mu);
-        if (ab > abs_bits(o.scale)) o.scale = from_bits(ab, F(0));
-        if (mono_key(mu) < mono_key(o.worst)) { o.worst = mu; o.widx = t * NU + ra; }
-        if (nan_key(ab, F(0))) o.bad = 1;
-      }
-    }
-    if (act && r < NU) Us[((size_t)t * NU + ra) * N + ai] = ul;
-    if (act && r < NX) Xo[((size_t)(t + 1) * NX + rr) * N + ai] = xn;
-    xl = xn;
-  }
-  if (row && (!(xl == xl) || fabs_(xl) > F(1e30))) o.bad = 1;
-  // combine the group's lanes: first (lowest index) most negative multiplier,
-  // largest |mu|, any flag
-#pragma unroll
-  for (int off = GS / 2; off > 0; off >>= 1) {
-    const F w2 = shfl_f(o.worst, lane ^ off);
-    const int i2 = __shfl_sync(FULL, o.widx, lane ^ off);
-    const F s2 = shfl_f(o.scale, lane ^ off);
-    const int b2i = __shfl_sync(FULL, o.bad, lane ^ off), o2 = __shfl_sync(FULL, o.out, lane ^ off);
-    const unsigned long long k1 = mono_key(o.worst), k2 = mono_key(w2);
-    if (i2 >= 0 && (o.widx < 0 || k2 < k1 || (k2 == k1 && i2 < o.widx))) {
-      o.worst = w2;
-      o.widx = i2;
-    }
-    if (abs_bits(s2) > abs_bits(o.scale)) o.scale = s2;
-    o.bad |= b2i;
-    o.out |= o2;
-  }
-  // the owner takes its group's result
-  const int gi = __popc(owners & ((1u << lane) - 1u));
-  const int from = (go ? gi : g) * GS;
-  EqpScan<F> res;
-  res.anum = 1; res.aden = 1; res.blk = -1; res.bside = 0;
-  res.worst = shfl_f(o.worst, from);
-  res.widx = __shfl_sync(FULL, o.widx, from);
-  res.scale = shfl_f(o.scale, from);
-  res.bad = __shfl_sync(FULL, o.bad, from);
-  res.out = __shfl_sync(FULL, o.out, from);
-  __syncwarp();
-  return res;
-}
+namespace tadmm {
 
 // Ratio test of the primal active set (Nocedal & Wright Alg. 16.3) for the step
 // p = us - u over the free inputs: smallest blocking ratio (clamped at 0), ties
@@ -1253,7 +814,7 @@ __device__ __forceinline__ void step_inputs(const AgentCtx<F, NX, NU, DP>& A, in
 // whatever number of lanes it serves.  Each lane's own sequence of working
 // sets, steps and multiplier tests is unchanged.
 // Returns ST_CONVERGED, ST_QP_FAIL or ST_NUMERIC.
-template <typename F, int NX, int NU, int DP, bool DI, bool COOP_EQP>
+template <typename F, int NX, int NU, int DP, bool DI>
 __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int start_kind, int as_max, F eps_rel,
                              unsigned long long& neqp, unsigned long long& nfact) {
   constexpr unsigned FULL = 0xffffffffu;
@@ -1293,10 +854,14 @@ __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int sta
   const bool lqr = has && start_kind == QP_LQR;
   if (__any_sync(FULL, lqr)) {
     int bad = 0;
-    refactor_sweep<F, NX, NU, DP, DI>(A, lqr, dirty, nfact, bad);
+    if constexpr (DI) {
+      bad = axis_round<F, NX, NU, DP>(A, lqr, dirty, nfact) & PASS_BAD;
+    } else {
+      refactor_sweep<F, NX, NU, DP>(A, lqr, dirty, nfact, bad);
+      if (lqr) bad |= eqp_solve<F, NX, NU, DP>(A).bad;
+    }
     if (lqr) {
-      const EqpScan<F> o = eqp_solve<F, NX, NU, DP, DI>(A);
-      if (bad || o.bad) {
+      if (bad) {
         status = ST_NUMERIC;
       } else {
         dirty = -1;
@@ -1325,25 +890,28 @@ __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int sta
     }
     if (!__any_sync(FULL, go)) break;
     int bad = 0;
-    refactor_sweep<F, NX, NU, DP, DI>(A, go, dirty, nfact, bad);
-    // few agents in this round: each takes its pass on a group of lanes
     EqpScan<F> o;
-    bool coop_pass = false;
-    if constexpr (COOP_EQP && DI && (std::is_same<F, double>::value || std::is_same<F, float>::value)) {
-      if (A.coop && __popc(__ballot_sync(FULL, go)) <= CoopShape<NX>::NG) {
-        o = eqp_coop<F, NX, NU, DP>(A, go);
-        coop_pass = true;
-      }
+    if constexpr (DI) {
+      const int found = axis_round<F, NX, NU, DP>(A, go, dirty, nfact);
+      o.anum = 1; o.aden = 1; o.blk = -1; o.bside = 0; o.worst = 0; o.widx = -1; o.scale = 1; o.bad = 0;
+      bad = found & PASS_BAD;
+      // the multipliers count only when nothing blocks the step
+      if (go && !bad && (found & PASS_OUT)) ratio_test<F, NX, NU, DP>(A, o);
+      const bool scan = go && !bad && (found & PASS_MULT) && (o.blk < 0 || (found & PASS_NAN));
+      mult_scan<F, NX, NU, DP>(A, scan, o);
+      o.out = 0;
+    } else {
+      refactor_sweep<F, NX, NU, DP>(A, go, dirty, nfact, bad);
+      if (go) o = eqp_solve<F, NX, NU, DP>(A);
     }
     if (go) {
       --as_max;
       ++neqp;
-      if (!coop_pass) o = eqp_solve<F, NX, NU, DP, DI>(A);
       if (bad || o.bad) {
         status = ST_NUMERIC;
       } else {
         dirty = -1;
-        if (o.out) ratio_test<F, NX, NU, DP>(A, o);
+        if (!DI && o.out) ratio_test<F, NX, NU, DP>(A, o);
         if (o.blk >= 0) {
           const F alpha = o.anum / o.aden;
           step_inputs<F, NX, NU, DP>(A, T, false, alpha);
@@ -1519,7 +1087,6 @@ __device__ __forceinline__ df64 step_rn(df64 u, df64 s, df64 v) { return u + s *
 // dmu; returns 1 on a non-finite value.
 template <typename F, int NX, int NU, int DP, bool DI>
 __device__ int eqp_direction(const AgentCtx<F, NX, NU, DP>& A, const F* hprev, F* dmu) {
-  constexpr int H = NX / 2;
   using CL = CacheLayout<NX, NU>;
   const Model<F, NX, NU>& Mo = *A.M;
   const int T = A.T, N = A.N, i = A.i;
@@ -1531,6 +1098,45 @@ __device__ int eqp_direction(const AgentCtx<F, NX, NU, DP>& A, const F* hprev, F
     return lin_term(base, A.k(AgentConst<NX, NU>::RHO), A.hv(t, r)) -
            lin_term(base, A.k(AgentConst<NX, NU>::RHO), hp);
   };
+  if constexpr (DI) {
+    // one axis after the other, on the axis words of the factor cache
+    using L = AxisCache;
+    const AxisView<F, NX, NU, DP, DP> V = axis_view<F, NX, NU, DP>(A);
+    const F a22 = Mo.A[DP][DP];  // 1, read so that the product below stays rounded
+    int bad = 0;
+    for (int a = 0; a < DP; ++a) {
+      F pp = dq(T, a), pv = dq(T, DP + a);
+      for (int t = T - 1; t >= 0; --t) {
+        const bool hd = V.held(A.W(t), a);
+        const F bp = fma(V.b2, pv, V.b1 * pp), g1 = V.C(t, L::G1, a), g2 = V.C(t, L::G2, a);
+        V.C(t, L::D, a) = hd ? bp : -(V.C(t, L::SI, a) * bp);
+        if (t >= 1) {
+          const F np = dq(t, a) + pp, nv = fma(a22, pv, V.dt * pp);
+          pp = hd ? np : fma(g1, bp, np);
+          pv = hd ? nv : fma(g2, bp, nv);
+        }
+      }
+      F xp = F(0), xv = F(0);
+      for (int t = 0; t < T; ++t) {
+        const uint32_t mask = A.W(t);
+        const bool hd = V.held(mask, a);
+        const F g1 = V.C(t, L::G1, a), g2 = V.C(t, L::G2, a), k = V.C(t, L::D, a);
+        const F u = hd ? F(0) : fma(g2, xv, fma(g1, xp, k));
+        xp = fma(V.b1, u, fma(V.dt, xv, xp));
+        xv = fma(V.b2, u, xv);
+        A.us(t, a) = u;
+        F d = F(0);
+        if (hd) {
+          // B' dlambda_{t+1} = (P_{t+1} B)' dx_{t+1} + B' dp_{t+1}
+          const F g = fma(g2, xv, fma(g1, xp, k));
+          d = ((mask >> a) & 1u) ? g : -g;
+        }
+        dmu[((size_t)t * NU + a) * N + i] = d;
+        if (!finite_(d) || !finite_(u)) bad = 1;
+      }
+    }
+    return bad;
+  }
   F pn[NX];
 #pragma unroll
   for (int r = 0; r < NX; ++r) pn[r] = dq(T, r);
@@ -1548,13 +1154,8 @@ __device__ int eqp_direction(const AgentCtx<F, NX, NU, DP>& A, const F* hprev, F
 #pragma unroll
     for (int a = 0; a < NU; ++a) {
       F acc = 0;
-      if constexpr (DI) {
-        acc = fma(Mo.B[0][0], pn[a], acc);
-        acc = fma(Mo.B[H][0], pn[H + a], acc);
-      } else {
 #pragma unroll
-        for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], pn[r], acc);
-      }
+      for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], pn[r], acc);
       bpn[a] = acc;
       sv[a] = (mask & (0x101u << a)) ? F(0) : acc;
     }
@@ -1650,7 +1251,8 @@ __device__ int homotopy_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, const 
     const bool go = !done && steps < as_max;
     if (!__any_sync(FULL, go)) break;
     int bad = 0;
-    refactor_sweep<F, NX, NU, DP, DI>(A, go, dirty, nfact, bad);
+    if constexpr (DI) bad = axis_round<F, NX, NU, DP, false>(A, go, dirty, nfact);
+    else refactor_sweep<F, NX, NU, DP>(A, go, dirty, nfact, bad);
     if (!go) continue;
     ++steps;
     ++neqp;
@@ -1754,7 +1356,7 @@ __device__ void homotopy_store(const AgentCtx<F, NX, NU, DP>& A, F* hprev, F* mu
 // x-update of agents i0, i0 + stride, ... of scenario s (none when in_scen is
 // false).  Every lane of the warp calls this; all lanes take the same number
 // of rounds, so that xupdate_agent always runs warp-wide.
-template <typename F, int NX, int NU, int DP, bool DI, bool COOP_EQP = false, bool HOMO = false>
+template <typename F, int NX, int NU, int DP, bool DI, bool HOMO = false>
 __device__ int xupdate_phase(const Dev<F>& D, const Model<F, NX, NU>& M, const ScenMeta& s, bool in_scen, int k,
                              int lvl_out, int i0, int stride, unsigned long long& neqp,
                              unsigned long long& nfact, F* kcs) {
@@ -1778,7 +1380,7 @@ __device__ int xupdate_phase(const Dev<F>& D, const Model<F, NX, NU>& M, const S
         res = homotopy_agent<F, NX, NU, DP, DI>(A, hh, D.hprev + s.as_off * DP, D.mu + s.as_off * NU,
                                                D.dmu + s.as_off * NU, as_max, neqp, nfact);
     }
-    const int r2 = xupdate_agent<F, NX, NU, DP, DI, COOP_EQP>(A, has && res == ST_CONVERGED, kind, as_max, eps,
+    const int r2 = xupdate_agent<F, NX, NU, DP, DI>(A, has && res == ST_CONVERGED, kind, as_max, eps,
                                                              neqp, nfact);
     if (res == ST_CONVERGED) res = r2;
     if constexpr (HOMO) {
@@ -2299,9 +1901,7 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
   }
 }
 
-// COOP_EQP: active-set rounds that serve at most CoopShape<NX>::NG agents of the
-// warp take their EQP pass on lane groups (eqp_coop, the same bits as eqp_solve).
-template <typename F, int NX, int NU, int DP, bool DI, bool COOP_EQP = false>
+template <typename F, int NX, int NU, int DP, bool DI>
 __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int* members, int G, GroupSm& gs,
                           GroupStage<F, DP>& st, F* sm, F* kcs) {
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -2367,7 +1967,7 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
                                             : idle_agent<F, NX, NU, DP>(M, kcs + tid, nt, D.coop);
       const int as_max = D.as_max > 0 ? D.as_max : 10 * s.T * NU + 10;
       const F eps = D.eps_rel > 0 ? F(D.eps_rel) : (sizeof(F) == 8 ? F(1e-12) : F(1e-5));
-      const int st = xupdate_agent<F, NX, NU, DP, DI, COOP_EQP>(A, has, start_kind_of(D, k), as_max, eps, neqp,
+      const int st = xupdate_agent<F, NX, NU, DP, DI>(A, has, start_kind_of(D, k), as_max, eps, neqp,
                                                                 nfact);
       if (has && st) atomicMax(&gs.flag[my_m], st);
     }

@@ -17,8 +17,6 @@ namespace tadmm {
 // ---------------------------------------------------------------------------
 // Register-budget variants of the persistent kernel (chosen by the autotuner):
 // (max threads per CTA, min resident CTAs per SM) for __launch_bounds__.
-// Variant 0, with no register cap, also runs small active-set rounds on lane
-// groups (COOP_EQP of run_group); the results are the same bits either way.
 template <int V> struct KVariant;
 template <> struct KVariant<0> { static constexpr int maxt = 256, minb = 1; };
 template <> struct KVariant<1> { static constexpr int maxt = 32, minb = 12; };
@@ -50,7 +48,7 @@ __global__ void __launch_bounds__(KVariant<V>::maxt, KVariant<V>::minb) k_batche
       const ScenMeta s = D.meta[sc];
       run_scenario<F, NX, NU, DP, DI>(D, M, s, sc, cs, sm, D.sm_pairs, kcs);
     } else {
-      run_group<F, NX, NU, DP, DI, (V == 0)>(D, M, D.gmem + b0, G, gs, gst, sm, kcs);
+      run_group<F, NX, NU, DP, DI>(D, M, D.gmem + b0, G, gs, gst, sm, kcs);
     }
   }
 }
@@ -81,7 +79,7 @@ __global__ void __launch_bounds__(32) k_xupdate(Dev<F> D, int sc, int k, int lvl
   const bool owns = (int)threadIdx.x < apw;
   const int i = blockIdx.x * apw + threadIdx.x;
   unsigned long long neqp = 0, nfact = 0;
-  const int st = xupdate_phase<F, NX, NU, DP, DI, true, HOMO>(D, M, s, owns, k, lvl_out, i, s.N, neqp, nfact, kcs);
+  const int st = xupdate_phase<F, NX, NU, DP, DI, HOMO>(D, M, s, owns, k, lvl_out, i, s.N, neqp, nfact, kcs);
   if (st && owns && i < s.N) atomicMax(flag, st);
   if (neqp) atomicAdd(&D.eqp[sc], neqp);
   if (nfact) atomicAdd(&D.fact[sc], nfact);
@@ -193,7 +191,7 @@ __global__ void __launch_bounds__(32) k_g_xupdate(Dev<F> D, GState G, const int3
   const int i = (int)(ga - s.agent_off), k = G.iter[sc];
   unsigned long long neqp = 0, nfact = 0;
   const int st =
-      xupdate_phase<F, NX, NU, DP, DI, true, HOMO>(D, M, s, in_scen, k, (k + 1) & 1, i, s.N, neqp, nfact, kcs);
+      xupdate_phase<F, NX, NU, DP, DI, HOMO>(D, M, s, in_scen, k, (k + 1) & 1, i, s.N, neqp, nfact, kcs);
   if (!in_scen) return;
   if (st) atomicMax(&G.fail[sc], st);
   if (neqp) atomicAdd(&D.eqp[sc], neqp);
@@ -758,17 +756,15 @@ int Impl<F, NX, NU, DP>::solve_batched(tadmm_handle* h, double tol, int max_iter
   return cuda_check(cudaGraphLaunch(h->gexec, st), "graph launch");
 }
 
-// Agents per warp of the per-phase x-update kernels: at most one per lane
-// group of the cooperative passes (CoopShape<NX>::NG: 8 in 2D, 4 in 3D), and
-// fewer, down to one, when there are not enough agents to give every SM four
-// warps.  Each of an SM's four sub-partitions issues FP64 instructions at its
-// own fixed rate whatever the number of active lanes, so a small agent count
-// (one large scenario) is spread over four warps per SM, one per
-// sub-partition, rather than packed into fewer warps; every owner can take its
-// EQP passes and refactorizations on a lane group.
+// Agents per warp of the per-phase x-update kernels: at most 8 in 2D and 4 in 3D,
+// whose axes fit the warp's lanes, and fewer, down to one, when there are not
+// enough agents to give every SM four warps.  Each of an SM's four sub-partitions
+// issues FP64 instructions at its own fixed rate whatever the number of active
+// lanes, so a small agent count (one large scenario) is spread over four warps
+// per SM, one per sub-partition, rather than packed into fewer warps.
 template <int NX>
 static int agents_per_warp(int64_t agents, int sm_count) {
-  int apw = CoopShape<NX>::NG;
+  int apw = NX <= 4 ? 8 : 4;
   while (apw > 1 && (int64_t)apw * sm_count * 4 > agents) apw /= 2;
   return apw;
 }

@@ -1,0 +1,61 @@
+"""The double integrator's per-axis recursions at the agent counts where the lane
+layout changes (one lane per axis holds 16 agents of a warp in 2D, 10 in 3D) and at
+the shortest horizons."""
+import numpy as np
+import pytest
+
+from instances import make_batch, random_scenario
+
+pytestmark = pytest.mark.gpu
+
+
+def _one(dp, N, T, seed):
+    return random_scenario(seed=seed, N=N, T=T, dp=dp, box=6.0, umax=0.6)
+
+
+def _run(b, **kw):
+    import paper_2602_15838_gb300 as tg
+    s = tg.Solver(b, **kw)
+    s.solve(0.0, 9)
+    out = s.solution()
+    cnt = s.counters()
+    s.close()
+    return out, cnt
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("dp,N,T", [(2, 1, 1), (2, 2, 2), (2, 16, 7), (2, 17, 7), (2, 32, 12), (3, 1, 1), (3, 10, 7),
+                                    (3, 11, 7), (3, 32, 9)])
+def test_axis_recursions(dp, N, T, precision):
+    """One lane per axis and one lane per agent give the same bits and counts, in
+    the batched and the graph mode; the general dense products give the same
+    working sets and, in float64, the same iterates to 1e-12 (nine iterations of
+    rounding of a few ulp of well conditioned stages)."""
+    import paper_2602_15838_gb300 as tg
+    b = _one(dp, N, T, seed=100 * dp + N)
+    ref, cref = _run(b, precision=precision, flags=tg.FLAG_NO_LANE_GROUPS)
+    for kw in (dict(), dict(threads_per_cta=32), dict(mode="graph"), dict(mode="graph", flags=tg.FLAG_NO_LANE_GROUPS)):
+        g, c = _run(b, precision=precision, **kw)
+        for k in ("X", "U", "theta", "W", "status", "iters"):
+            assert np.array_equal(g[k], ref[k]), (kw, k)
+        assert np.array_equal(c["eqp"], cref["eqp"]) and np.array_equal(c["fact"], cref["fact"]), kw
+    if precision == 64:
+        d, cd = _run(b, flags=tg.FLAG_NO_STRUCTURE)
+        assert np.array_equal(d["W"], ref["W"]) and np.array_equal(cd["eqp"], cref["eqp"])
+        for k in ("X", "U", "theta"):
+            assert np.abs(d[k] - ref[k]).max(initial=0.0) <= 1e-12 * max(1.0, np.abs(ref[k]).max(initial=0.0)), k
+
+
+def test_large_magnitudes_and_held_multipliers():
+    """Weights and goals far from one: the float32 sign test of the multipliers
+    must hand over to float64 where its numbers leave float32's range, and the
+    result is the one of the dense products."""
+    import paper_2602_15838_gb300 as tg
+    b = _one(2, 6, 10, seed=5)
+    for f in (1e-30, 1e25):
+        c = make_batch([dict(N=6, T=10, x_init=b.x_init, x_ref=b.x_ref, a=b.a, w0=b.w0, d=0.4, rho=f, umax=0.6, c=None)],
+                       dp=2, dt=0.1, umax=0.6, q_pos=f, q_vel=0.1 * f, r=0.1 * f)
+        g, cg = _run(c)
+        d, cd = _run(c, flags=tg.FLAG_NO_STRUCTURE)
+        assert np.array_equal(g["W"], d["W"]) and np.array_equal(cg["eqp"], cd["eqp"])
+        assert np.abs(g["X"] - d["X"]).max() <= 1e-12 * np.abs(d["X"]).max()
