@@ -69,9 +69,11 @@ WORKLOAD_SOLVES, WORKLOAD_SCEN_ITERS = 194, 1955163
 WORKLOAD_SOLVES_PER_SCEN_ITER = WORKLOAD_SOLVES / WORKLOAD_SCEN_ITERS
 # algorithmic flops per unit: pair-step, EQP stage, factorized stage.  The double
 # integrator's stages fall apart into one two-state, one-input recursion per axis:
-# 26 flops of a pass and 35 of a factorization each (its zeros are not counted)
-FLOPS_2D = (30.0, 52.0, 70.0)       # nx = 4, nu = 2
-FLOPS_3D = (41.0, 78.0, 105.0)      # nx = 6, nu = 3
+# 26 flops of a pass and 35 of a factorization each (its zeros are not counted).
+# A pair-step: the projection (differences, product, step) and its term in either
+# agent's sum; the kernel forms them in FP64 only for the pairs that push
+FLOPS_2D = (16.0, 52.0, 70.0)       # nx = 4, nu = 2
+FLOPS_3D = (23.0, 78.0, 105.0)      # nx = 6, nu = 3
 FLOPS_PAIRSTEP, FLOPS_EQP_STAGE, FLOPS_FACT_STAGE = FLOPS_2D
 COUNTERS_FILE = os.path.join(ROOT, "profiles", "k_batched_mixed4096_counters.txt")
 
@@ -659,7 +661,7 @@ def other_workloads(tg, torch, args, peaks):
     row["ms_per_iteration_plain"] = _event_ms(torch, lambda: s.solve(0.0, 20), reps=2) / 20
     s.close()
     row["note"] = ("one scenario of 130816 pairs x 40 steps; the FP64 fraction counts algorithmic flops "
-                   "(41 per pair-step, 78 per EQP stage, 105 per factorized stage) over the measured FP64 peak")
+                   "(23 per pair-step, 78 per EQP stage, 105 per factorized stage) over the measured FP64 peak")
     out["swarm3d_512_agents"] = row
     # 64 scenarios x 16 agents, T = 30: solve, active-set polish and implicit-KKT backward
     b = make_workload("diff", n_scen=64)

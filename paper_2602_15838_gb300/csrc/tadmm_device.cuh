@@ -1759,10 +1759,16 @@ constexpr int kGroupPairs = kGroupMax * (kGroupMax - 1) / 2;
 
 template <typename F, int DP>
 struct GroupStage {
-  uint32_t pair[kGroupPairs];   // flattened agent indices fi | fj << 8 of every member pair
+  // flattened agent indices of every member pair and its place among either
+  // agent's partners: fi | fj << 8 | place at i << 16 | place at j << 24
+  uint32_t pair[kGroupPairs];
   uint8_t mem[kGroupPairs];     // member of every flattened pair
   F pos[DP][kGroupMax];         // positions p^{k+1} of the group's agents at the current step
   F sxs[DP][kGroupMax];         // over-relaxation: agent parts s^k of the consensus copies at that step
+  float posf[DP][kGroupMax];    // float64: the positions for the float32 test
+  uint32_t on[kGroupMax];       // places of the agent's partners with a coupling weight at the current step
+  uint16_t list[kGroupPairs];   // float64: pairs of the current step that need the projection
+  int count;                    // their number
 };
 
 struct GroupSm {
@@ -1773,16 +1779,46 @@ struct GroupSm {
   int active[kGroupMax];
   int flag[kGroupMax];
   int need[kGroupMax];
-  unsigned long long rb[kGroupMax];  // primal residual key (unrelaxed: max |theta' - theta|, a bound)
+  unsigned long long rb[kGroupMax];  // primal residual key (unrelaxed: max |theta' - theta|, a bound); keys start at zero's own
   unsigned long long sb[kGroupMax];
   unsigned long long rx[kGroupMax];  // exact primal residual key from the lazy pass
   unsigned long long cnt[kGroupMax][2];
   double rho[kGroupMax];    // current penalty per member (residual balancing)
   double scale[kGroupMax];  // this iteration's penalty factor per member
   int rhoc[kGroupMax];      // penalty changes per member
+  float df[kGroupMax];      // float64: the member's separation for the float32 test
   int adapt[kGroupMax];     // member's penalty changed this iteration
   int G, nA, nP, T, any, anyad;
 };
+
+// Place of partner j (coupled by scenario-local pair `pair`) among agent i's
+// partners in increasing order: the order of for_partners.
+template <typename F>
+__device__ __forceinline__ int partner_place(const Dev<F>& D, const ScenMeta& s, int i, int j, int pair) {
+  if (!s.sparse) return j < i ? j : j - 1;
+  int e = D.adj_ptr[s.agent_off + i];
+  const int e0 = e;
+  while ((D.adj[e] & 0x7FFFFFFF) != pair) ++e;
+  return e - e0;
+}
+
+// Calls ea(pair, first) for agent i's partners at the places in `on`, in
+// increasing order (for_partners without the others).
+template <typename F, class EA>
+__device__ __forceinline__ void for_places(const Dev<F>& D, const ScenMeta& s, int i, uint32_t on, EA&& ea) {
+  const int e0 = s.sparse ? D.adj_ptr[s.agent_off + i] : 0;
+  for (; on; on &= on - 1) {
+    const int b = __ffs(on) - 1;
+    if (s.sparse) {
+      const uint32_t ent = (uint32_t)D.adj[e0 + b];
+      ea((int)(ent & 0x7FFFFFFFu), (ent >> 31) == 0u);
+    } else {
+      const int j = b < i ? b : b + 1;
+      const bool first = i < j;
+      ea(first ? pair_index(s.N, i, j) : pair_index(s.N, j, i), first);
+    }
+  }
+}
 
 // Member owning flattened index u given exclusive prefix sums off[0..G].
 __device__ __forceinline__ int member_of(const int* off, int G, int u) {
@@ -1836,7 +1872,7 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
       const size_t q = s.ps_off + (size_t)tm1 * P + pair;
       const F* a = D.a + s.ps_off * DP;
       const uint32_t fij = st.pair[u];
-      const int fi = fij & 0xFF, fj = fij >> 8;
+      const int fi = fij & 0xFF, fj = (fij >> 8) & 0xFF;
       const F th = D.theta[(size_t)tk * D.tot_ps + q];
       const F ph = D.phi[q];
       F av[DP];
@@ -1901,6 +1937,169 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
   }
 }
 
+// Consensus projection, dual update and gather of a group, step by step: the
+// arithmetic of pair_phase and gather_phase.  The step's positions and the pair
+// table are read from shared memory; the next step's positions, and the operands
+// of each batch of kPairBatch pairs, are loaded ahead of their use.
+//
+// Few pairs push at a time (a few in a hundred on the mixed workload): where
+// theta^k = 0 and the halfspace holds, theta^{k+1} = 0, and the pair adds nothing
+// to the residual or to any agent's sum.  In float64 these pairs are found by a
+// float32 value of d - a'(p_i - p_j) with a margin over its error (positions and
+// normals cut to 24 bits: 2^-23 of each, four roundings; the margin is 2^-19 of
+// the sizes' sum), the others are listed and take the projection, full lanes at a
+// time, and each agent sums the partners that it has a weight with, in their
+// order.  The values are those of the plain sweep: a left-out term is a zero.
+// What bounds it is then the 24 + 8 bytes per pair-step and their latency, no
+// longer 11 FP64 instructions per 32 pair-steps: the 4096-scenario mixed batch
+// over 500 iterations went from 543 to 356 ms, 256 scenarios over 30 iterations
+// with the host's copies from 63 to 59 ms, float32 (no test needed, the same
+// sparse sums) over 1024 scenarios and 200 iterations from 69 to 53 ms.
+template <typename F, int NX, int DP>
+__device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st, F* smE, F* smA, int my_m, int my_i,
+                            int xl, int tk, int tkp1) {
+  constexpr bool kTest = std::is_same<F, double>::value;
+  const int tid = threadIdx.x, nt = blockDim.x, nP = gs.nP, T = gs.T;
+  const bool mine = my_m >= 0 && gs.active[my_m];
+  const F* const th_k = D.theta + (size_t)tk * D.tot_ps;
+  F* const th_n = D.theta + (size_t)tkp1 * D.tot_ps;
+  const F* Xmine = nullptr;
+  int Nmine = 1;
+  F pnext[DP];
+  if (mine) {
+    const ScenMeta& s = gs.meta[my_m];
+    Xmine = D.X + (size_t)(xl ^ 1) * D.tot_xs * NX + s.xs_off * NX;
+    Nmine = s.N;
+#pragma unroll
+    for (int c = 0; c < DP; ++c) pnext[c] = Xmine[((size_t)NX + c) * Nmine + my_i];
+  }
+  // projection of pair u of member m: theta^{k+1}, the residual bound and, where
+  // it is not zero, the coupling weight 2 theta^{k+1} - theta^k of both agents
+  auto project = [&](int u, int m, const F (&av)[DP], F th, F* tn_out) {
+    const uint32_t fij = st.pair[u];
+    const int fi = fij & 0xFF, fj = (fij >> 8) & 0xFF;
+    F g = F(gs.meta[m].d);  // d - a'(p_i - p_j)
+#pragma unroll
+    for (int c = 0; c < DP; ++c) g = fma(-av[c], st.pos[c][fi] - st.pos[c][fj], g);
+    F tn = fma(g, F(0.5), th);
+    if (sign_set(tn)) tn = F(0);
+    *tn_out = tn;
+    if (tn != F(0) || th != F(0)) {
+      smE[u] = fma(F(2), tn, -th);
+#pragma unroll
+      for (int c = 0; c < DP; ++c) smA[c * nP + u] = av[c];
+      atomicOr(&st.on[fi], 1u << ((fij >> 16) & 0xFF));
+      atomicOr(&st.on[fj], 1u << (fij >> 24));
+      // max |theta' - theta| bounds the primal residual r = max |(theta' - theta) a_c|
+      // (|a| = 1): r <= it <= sqrt(dp) r; the exact r is formed in the lazy pass
+      const unsigned long long v = abs_bits(tn - th);
+      if (v > gs.rb[m]) atomicMax(&gs.rb[m], v);
+    }
+  };
+  for (int tm1 = 0; tm1 < T; ++tm1) {
+    if (mine) {
+#pragma unroll
+      for (int c = 0; c < DP; ++c) {
+        st.pos[c][tid] = pnext[c];
+        if constexpr (kTest) st.posf[c][tid] = near_f32(pnext[c]);
+      }
+    }
+    __syncthreads();
+    for (int ub = tid; ub - tid < nP; ub += kPairBatch * nt) {
+      F av[kPairBatch][DP], thv[kPairBatch];
+      int mk[kPairBatch];
+      int64_t qk[kPairBatch];
+#pragma unroll
+      for (int b = 0; b < kPairBatch; ++b) {
+        const int u = ub + b * nt;
+        mk[b] = -1;
+        if (u < nP) {
+          const int m = st.mem[u];
+          if (gs.active[m]) {
+            mk[b] = m;
+            const ScenMeta& s = gs.meta[m];
+            const int P = s.P, pair = u - gs.poff[m];
+            const F* a = D.a + s.ps_off * DP;
+#pragma unroll
+            for (int c = 0; c < DP; ++c) av[b][c] = a[((size_t)tm1 * DP + c) * P + pair];
+            qk[b] = s.ps_off + (int64_t)tm1 * P + pair;
+            thv[b] = th_k[qk[b]];
+          }
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < kPairBatch; ++b) {
+        const int u = ub + b * nt, m = mk[b];
+        if constexpr (kTest) {
+          bool want = false;
+          if (m >= 0) {
+            const uint32_t fij = st.pair[u];
+            const int fi = fij & 0xFF, fj = (fij >> 8) & 0xFF;
+            float g = gs.df[m], size = fabsf(g);
+#pragma unroll
+            for (int c = 0; c < DP; ++c) {
+              const float af = near_f32(av[b][c]), pi = st.posf[c][fi], pj = st.posf[c][fj];
+              g = fmaf(-af, pi - pj, g);
+              size = fmaf(fabsf(af), fabsf(pi) + fabsf(pj), size);
+            }
+            want = !(thv[b] == F(0) && g < -fmaf(size, 0x1p-19f, 1e-17f));
+            if (!want) th_n[qk[b]] = F(0);
+          }
+          const unsigned ball = __ballot_sync(0xffffffffu, want);
+          if (ball) {
+            int base = 0;
+            if ((tid & 31) == 0) base = atomicAdd(&st.count, __popc(ball));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (want) st.list[base + __popc(ball & ((1u << (tid & 31)) - 1u))] = (uint16_t)u;
+          }
+        } else {
+          if (m >= 0) project(u, m, av[b], thv[b], &th_n[qk[b]]);
+        }
+      }
+    }
+    __syncthreads();
+    if constexpr (kTest) {
+      const int n = st.count;
+      for (int l = tid; l < n; l += nt) {
+        const int u = st.list[l], m = st.mem[u];
+        const ScenMeta& s = gs.meta[m];
+        const int P = s.P, pair = u - gs.poff[m];
+        const F* a = D.a + s.ps_off * DP;
+        F av[DP];
+#pragma unroll
+        for (int c = 0; c < DP; ++c) av[c] = a[((size_t)tm1 * DP + c) * P + pair];
+        const int64_t q = s.ps_off + (int64_t)tm1 * P + pair;
+        project(u, m, av, th_k[q], &th_n[q]);
+      }
+      __syncthreads();
+      if (tid == 0) st.count = 0;
+    }
+    if (mine && tm1 + 1 < T) {
+#pragma unroll
+      for (int c = 0; c < DP; ++c) pnext[c] = Xmine[((size_t)(tm1 + 2) * NX + c) * Nmine + my_i];
+    }
+    if (mine) {
+      const ScenMeta& s = gs.meta[my_m];
+      const int N = s.N, i = my_i, base = gs.poff[my_m];
+      F acc[DP];
+#pragma unroll
+      for (int c = 0; c < DP; ++c) acc[c] = F(agent_nc(D, s, i)) * st.pos[c][tid];
+      for_places(D, s, i, st.on[tid], [&](int lp, bool first) {
+        const int pair = base + lp;
+        F e = smE[pair];
+        if (!first) e = -e;
+#pragma unroll
+        for (int c = 0; c < DP; ++c) acc[c] = fma(e, smA[c * nP + pair], acc[c]);
+      });
+      st.on[tid] = 0;
+      F* h = D.h + s.as_off * DP;
+#pragma unroll
+      for (int c = 0; c < DP; ++c) h[((size_t)tm1 * DP + c) * N + i] = acc[c];
+    }
+  }
+  __syncthreads();
+}
+
 template <typename F, int NX, int NU, int DP, bool DI>
 __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int* members, int G, GroupSm& gs,
                           GroupStage<F, DP>& st, F* sm, F* kcs) {
@@ -1912,15 +2111,18 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
     gs.active[tid] = 1;
     gs.flag[tid] = 0;
     gs.need[tid] = 0;
-    gs.rb[tid] = 0;
-    gs.sb[tid] = 0;
-    gs.rx[tid] = 0;
+    gs.rb[tid] = ord_bits(F(0));
+    gs.sb[tid] = ord_bits(F(0));
+    gs.rx[tid] = ord_bits(F(0));
     gs.cnt[tid][0] = 0;
     gs.cnt[tid][1] = 0;
     gs.rho[tid] = gs.meta[tid].rho;
     gs.rhoc[tid] = 0;
     gs.adapt[tid] = 0;
+    gs.df[tid] = near_f32(gs.meta[tid].d);
   }
+  if (tid < kGroupMax) st.on[tid] = 0;
+  if (tid == 0) st.count = 0;
   __syncthreads();
   if (tid == 0) {
     int a = 0, p = 0;
@@ -1942,9 +2144,11 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
   const int nA = gs.nA, nP = gs.nP, T = gs.T;
   for (int u = tid; u < nP; u += nt) {
     const int m = member_of(gs.poff, G, u);
-    const int pk = D.pairs[gs.meta[m].pair_off + (u - gs.poff[m])];
+    const ScenMeta& s = gs.meta[m];
+    const int pair = u - gs.poff[m], pk = D.pairs[s.pair_off + pair], i = pk & 0xFFFF, j = pk >> 16;
     st.mem[u] = (uint8_t)m;
-    st.pair[u] = (uint32_t)(gs.aoff[m] + (pk & 0xFFFF)) | ((uint32_t)(gs.aoff[m] + (pk >> 16)) << 8);
+    st.pair[u] = (uint32_t)(gs.aoff[m] + i) | ((uint32_t)(gs.aoff[m] + j) << 8) |
+                 ((uint32_t)partner_place(D, s, i, j, pair) << 16) | ((uint32_t)partner_place(D, s, j, i, pair) << 24);
   }
   __syncthreads();
   // the lane's agent (fixed for the whole run)
@@ -1980,101 +2184,11 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
       D.cur_lvl[sc] = xl | (tk << 1);
     }
     __syncthreads();
-    // fused consensus projection / dual update and gather, step by step; the
-    // step's positions and the pair table are read from shared memory.  The
-    // next step's positions, and the operands of each batch of kPairBatch
-    // pairs, are loaded ahead of their use so that the load latency overlaps
-    // the arithmetic.
+    // fused consensus projection / dual update and gather, step by step
     if (D.relax) {
       group_relaxed_sweep<F, NX, DP>(D, gs, st, smE, smA, my_m, my_i, xl, tk, tkp1);
     } else {
-      const bool mine = my_m >= 0 && gs.active[my_m];
-      const F* Xmine = nullptr;
-      int Nmine = 1;
-      F pnext[DP];
-      if (mine) {
-        const ScenMeta& s = gs.meta[my_m];
-        Xmine = D.X + (size_t)(xl ^ 1) * D.tot_xs * NX + s.xs_off * NX;
-        Nmine = s.N;
-#pragma unroll
-        for (int c = 0; c < DP; ++c) pnext[c] = Xmine[((size_t)NX + c) * Nmine + my_i];
-      }
-      for (int tm1 = 0; tm1 < T; ++tm1) {
-        if (mine) {
-#pragma unroll
-          for (int c = 0; c < DP; ++c) st.pos[c][tid] = pnext[c];
-        }
-        __syncthreads();
-        for (int ub = tid; ub < nP; ub += kPairBatch * nt) {
-          F av[kPairBatch][DP], thv[kPairBatch];
-          int mk[kPairBatch];
-#pragma unroll
-          for (int b = 0; b < kPairBatch; ++b) {
-            const int u = ub + b * nt;
-            mk[b] = -1;
-            if (u < nP) {
-              const int m = st.mem[u];
-              if (gs.active[m]) {
-                mk[b] = m;
-                const ScenMeta& s = gs.meta[m];
-                const int P = s.P, pair = u - gs.poff[m];
-                const F* a = D.a + s.ps_off * DP;
-#pragma unroll
-                for (int c = 0; c < DP; ++c) av[b][c] = a[((size_t)tm1 * DP + c) * P + pair];
-                thv[b] = D.theta[(size_t)tk * D.tot_ps + s.ps_off + (size_t)tm1 * P + pair];
-              }
-            }
-          }
-#pragma unroll
-          for (int b = 0; b < kPairBatch; ++b) {
-            if (mk[b] < 0) continue;
-            const int u = ub + b * nt, m = mk[b];
-            const ScenMeta& s = gs.meta[m];
-            const int P = s.P, pair = u - gs.poff[m];
-            const uint32_t fij = st.pair[u];
-            const int fi = fij & 0xFF, fj = fij >> 8;
-            F g = F(s.d);  // d - a'(p_i - p_j)
-#pragma unroll
-            for (int c = 0; c < DP; ++c) {
-              const F avc = av[b][c];
-              smA[c * nP + u] = avc;
-              g = fma(-avc, st.pos[c][fi] - st.pos[c][fj], g);
-            }
-            const F th = thv[b];
-            F tn = fma(g, F(0.5), th);
-            if (sign_set(tn)) tn = F(0);
-            D.theta[(size_t)tkp1 * D.tot_ps + s.ps_off + (size_t)tm1 * P + pair] = tn;
-            smE[u] = fma(F(2), tn, -th);
-            // max |theta' - theta| bounds the primal residual r = max |(theta' - theta) a_c|
-            // (|a| = 1): r <= it <= sqrt(dp) r; the exact r is formed in the lazy pass
-            const unsigned long long v = abs_bits(tn - th);
-            if (v > gs.rb[m]) atomicMax(&gs.rb[m], v);
-          }
-        }
-        __syncthreads();
-        if (mine && tm1 + 1 < T) {
-#pragma unroll
-          for (int c = 0; c < DP; ++c) pnext[c] = Xmine[((size_t)(tm1 + 2) * NX + c) * Nmine + my_i];
-        }
-        if (mine) {
-          const ScenMeta& s = gs.meta[my_m];
-          const int N = s.N, i = my_i, base = gs.poff[my_m];
-          F acc[DP];
-#pragma unroll
-          for (int c = 0; c < DP; ++c) acc[c] = F(agent_nc(D, s, i)) * st.pos[c][tid];
-          for_partners(D, s, i, [&](int lp, bool first) {
-            const int pair = base + lp;
-            F e = smE[pair];
-            if (!first) e = -e;
-#pragma unroll
-            for (int c = 0; c < DP; ++c) acc[c] = fma(e, smA[c * nP + pair], acc[c]);
-          });
-          F* h = D.h + s.as_off * DP;
-#pragma unroll
-          for (int c = 0; c < DP; ++c) h[((size_t)tm1 * DP + c) * N + i] = acc[c];
-        }
-        __syncthreads();
-      }
+      group_sweep<F, NX, DP>(D, gs, st, smE, smA, my_m, my_i, xl, tk, tkp1);
     }
     // primal residual tests on the bound, then the exact primal and the dual
     // residual in a lazy pass only where they decide (the over-relaxed sweep has
@@ -2148,9 +2262,9 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
           }
         }
       }
-      gs.rb[tid] = 0;
-      gs.sb[tid] = 0;
-      gs.rx[tid] = 0;
+      gs.rb[tid] = ord_bits(F(0));
+      gs.sb[tid] = ord_bits(F(0));
+      gs.rx[tid] = ord_bits(F(0));
     }
     __syncthreads();
     if (tid == 0) {

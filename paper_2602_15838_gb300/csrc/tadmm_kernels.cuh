@@ -705,7 +705,8 @@ int Impl<F, NX, NU, DP>::max_ctas_per_sm(int tpc, int variant, const tadmm_handl
   if (tpc > variant_maxt(variant)) return 0;
   const size_t smem = (h ? fused_smem_bytes<F, DP>(h, nullptr) : 0) + agent_const_bytes<F, NX, NU>(tpc);
   const void* kfn = batched_kernel<F, NX, NU, DP>(variant, h ? h->di != 0 : false);
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // 48 KB without it, the static part (about 11 KB) included
+  if (smem > 32 * 1024) cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kfn, tpc, smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
