@@ -1842,7 +1842,7 @@ __device__ __forceinline__ int member_of(const int* off, int G, int u) {
 // formed in this sweep.
 template <typename F, int NX, int DP>
 __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st, F* smE, F* smA,
-                                    int my_m, int my_i, int xl, int tk, int tkp1) {
+                                    int my_a, int my_m, int my_i, int xl, int tk, int tkp1) {
   const int tid = threadIdx.x, nt = blockDim.x, nP = gs.nP, T = gs.T;
   const F al = F(D.alpha), om = F(1.0 - D.alpha);
   const bool mine = my_m >= 0 && gs.active[my_m];
@@ -1859,8 +1859,8 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
     if (mine) {
 #pragma unroll
       for (int c = 0; c < DP; ++c) {
-        st.pos[c][tid] = Xm[((size_t)(tm1 + 1) * NX + c) * Nm + my_i];
-        st.sxs[c][tid] = Sm[((size_t)tm1 * DP + c) * Nm + my_i];
+        st.pos[c][my_a] = Xm[((size_t)(tm1 + 1) * NX + c) * Nm + my_i];
+        st.sxs[c][my_a] = Sm[((size_t)tm1 * DP + c) * Nm + my_i];
       }
     }
     __syncthreads();
@@ -1916,7 +1916,7 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
       F sn[DP], acc[DP];
 #pragma unroll
       for (int c = 0; c < DP; ++c) {
-        sn[c] = fma(al, st.pos[c][tid], om * st.sxs[c][tid]);
+        sn[c] = fma(al, st.pos[c][my_a], om * st.sxs[c][my_a]);
         acc[c] = nc * sn[c];
       }
       for_partners(D, s, i, [&](int lp, bool first) {
@@ -1956,8 +1956,8 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
 // with the host's copies from 63 to 59 ms, float32 (no test needed, the same
 // sparse sums) over 1024 scenarios and 200 iterations from 69 to 53 ms.
 template <typename F, int NX, int DP>
-__device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st, F* smE, F* smA, int my_m, int my_i,
-                            int xl, int tk, int tkp1) {
+__device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st, F* smE, F* smA, int my_a, int my_m,
+                            int my_i, int xl, int tk, int tkp1) {
   constexpr bool kTest = std::is_same<F, double>::value;
   const int tid = threadIdx.x, nt = blockDim.x, nP = gs.nP, T = gs.T;
   const bool mine = my_m >= 0 && gs.active[my_m];
@@ -2000,8 +2000,8 @@ __device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st,
     if (mine) {
 #pragma unroll
       for (int c = 0; c < DP; ++c) {
-        st.pos[c][tid] = pnext[c];
-        if constexpr (kTest) st.posf[c][tid] = near_f32(pnext[c]);
+        st.pos[c][my_a] = pnext[c];
+        if constexpr (kTest) st.posf[c][my_a] = near_f32(pnext[c]);
       }
     }
     __syncthreads();
@@ -2083,15 +2083,15 @@ __device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st,
       const int N = s.N, i = my_i, base = gs.poff[my_m];
       F acc[DP];
 #pragma unroll
-      for (int c = 0; c < DP; ++c) acc[c] = F(agent_nc(D, s, i)) * st.pos[c][tid];
-      for_places(D, s, i, st.on[tid], [&](int lp, bool first) {
+      for (int c = 0; c < DP; ++c) acc[c] = F(agent_nc(D, s, i)) * st.pos[c][my_a];
+      for_places(D, s, i, st.on[my_a], [&](int lp, bool first) {
         const int pair = base + lp;
         F e = smE[pair];
         if (!first) e = -e;
 #pragma unroll
         for (int c = 0; c < DP; ++c) acc[c] = fma(e, smA[c * nP + pair], acc[c]);
       });
-      st.on[tid] = 0;
+      st.on[my_a] = 0;
       F* h = D.h + s.as_off * DP;
 #pragma unroll
       for (int c = 0; c < DP; ++c) h[((size_t)tm1 * DP + c) * N + i] = acc[c];
@@ -2151,9 +2151,15 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
                  ((uint32_t)partner_place(D, s, i, j, pair) << 16) | ((uint32_t)partner_place(D, s, j, i, pair) << 24);
   }
   __syncthreads();
-  // the lane's agent (fixed for the whole run)
-  const int my_m = tid < nA ? member_of(gs.aoff, G, tid) : -1;
-  const int my_i = tid < nA ? tid - gs.aoff[my_m] : 0;
+  // The lane's agent (fixed for the whole run).  A warp takes as many agents as
+  // have their axes fit its lanes: its passes then go one axis per lane, which
+  // costs each warp half (2D) or a third (3D) of a pass with whole agents, on a
+  // sub-partition of its own.  With fewer warps than that they are shared evenly.
+  const int nw = nt >> 5, per = max((nA + nw - 1) / nw, min(nA, 32 / DP));
+  const int slot = (tid & 31) < per ? (tid >> 5) * per + (tid & 31) : nA;
+  const int my_a = slot < nA ? slot : -1;  // in the group
+  const int my_m = my_a >= 0 ? member_of(gs.aoff, G, my_a) : -1;
+  const int my_i = my_a >= 0 ? my_a - gs.aoff[my_m] : 0;
   unsigned long long neqp = 0, nfact = 0;
   F* smE = sm;
   F* smA = sm + nP;
@@ -2186,9 +2192,9 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
     __syncthreads();
     // fused consensus projection / dual update and gather, step by step
     if (D.relax) {
-      group_relaxed_sweep<F, NX, DP>(D, gs, st, smE, smA, my_m, my_i, xl, tk, tkp1);
+      group_relaxed_sweep<F, NX, DP>(D, gs, st, smE, smA, my_a, my_m, my_i, xl, tk, tkp1);
     } else {
-      group_sweep<F, NX, DP>(D, gs, st, smE, smA, my_m, my_i, xl, tk, tkp1);
+      group_sweep<F, NX, DP>(D, gs, st, smE, smA, my_a, my_m, my_i, xl, tk, tkp1);
     }
     // primal residual tests on the bound, then the exact primal and the dual
     // residual in a lazy pass only where they decide (the over-relaxed sweep has
