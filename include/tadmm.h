@@ -102,8 +102,10 @@ typedef struct {
   /* Heterogeneous agents (an extension: the paper's agents share one model).
    * NULL (both): every agent has A, B above.  Otherwise per-agent dynamics
    * A_agent [sum N][nx][nx] and B_agent [sum N][nx][nu], row-major, agents in
-   * scenario order; the input box stays shared.  The products are then the
-   * dense ones; not with TADMM_FLAG_DOUBLE_FLOAT (EINVAL). */
+   * scenario order; the input box stays shared.  Models of the form
+   * A = [[I, dt I], [0, a22 I]], B = [[b1 I], [b2 I]] keep the structured
+   * products, others take the dense ones; not with TADMM_FLAG_DOUBLE_FLOAT
+   * (EINVAL). */
   const double* A_agent;
   const double* B_agent;
 } tadmm_batch;

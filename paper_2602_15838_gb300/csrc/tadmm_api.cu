@@ -190,6 +190,41 @@ static bool is_double_integrator(const tadmm_batch* b) {
   return true;
 }
 
+// The same for per-agent models, each with its own coefficients and a factor
+// on the velocity: A = [[I, dt I], [0, a22 I]].
+static bool agents_separable(const tadmm_batch* b, int64_t na) {
+  const int nx = b->nx, nu = b->nu, H = nx / 2;
+  if (nu != H) return false;
+  for (int64_t i = 0; i < na; ++i) {
+    const double *A = b->A_agent + i * nx * nx, *B = b->B_agent + i * nx * nu;
+    for (int r = 0; r < nx; ++r) {
+      for (int c = 0; c < nx; ++c) {
+        double want = 0.0;
+        if (r == c) want = r < H ? 1.0 : A[H * nx + H];
+        if (r < H && c == r + H) want = A[H];
+        if (A[r * nx + c] != want) return false;
+      }
+      for (int c = 0; c < nu; ++c)
+        if (B[r * nu + c] != (c == r % H ? B[(r / H) * H * nu] : 0.0)) return false;
+    }
+  }
+  return true;
+}
+
+// Which products the handle's kernels take for the batch's dynamics.
+static void set_structure(tadmm_handle* h, const tadmm_batch* b, int64_t na) {
+  const bool on = !(h->opt.flags & TADMM_FLAG_NO_STRUCTURE);
+  const int di = (on && !h->hetero && is_double_integrator(b)) ? 1 : 0;
+  const int ax = (di || (on && h->hetero && agents_separable(b, na))) ? 1 : 0;
+  if (ax != h->ax) {  // captured graphs hold the other kernels
+    if (h->gexec) cudaGraphExecDestroy(h->gexec);
+    if (h->wexec) cudaGraphExecDestroy(h->wexec);
+    h->gexec = h->wexec = nullptr;
+  }
+  h->di = di;
+  h->ax = ax;
+}
+
 static void free_all(tadmm_handle* h) {
   if (!h) return;
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
@@ -334,7 +369,6 @@ extern "C" int tadmm_create(const tadmm_batch* b, const tadmm_options* opt, tadm
   h->cps = o.ctas_per_sm;
   h->variant = o.kernel_variant;
   h->hetero = b->A_agent ? 1 : 0;
-  h->di = (!(o.flags & TADMM_FLAG_NO_STRUCTURE) && !h->hetero && is_double_integrator(b)) ? 1 : 0;
   h->N.assign(b->N, b->N + b->n_scen);
   h->T.assign(b->T, b->T + b->n_scen);
   h->meta_h.resize(b->n_scen);
@@ -396,6 +430,7 @@ extern "C" int tadmm_create(const tadmm_batch* b, const tadmm_options* opt, tadm
       lpo += m.P;
     }
   }
+  set_structure(h, b, h->tot_agents);
   // processing order of the persistent kernel: largest estimated work first
   std::vector<int32_t> order(b->n_scen);
   std::iota(order.begin(), order.end(), 0);
@@ -554,6 +589,7 @@ extern "C" int tadmm_update(tadmm_handle* h, const tadmm_batch* b, void* stream)
     return set_error(TADMM_EINVAL, "update: batch shape differs from the handle");
   int rc = validate(b, h);
   if (rc) return rc;
+  set_structure(h, b, h->tot_agents);
   return upload_inputs(h, b, (cudaStream_t)stream);
 }
 

@@ -1,9 +1,10 @@
-// The x-update's equality-constrained solves for the double integrator (included
+// The x-update's equality-constrained solves for axis-separable models (included
 // by tadmm_device.cuh, after the agent context).
 //
-// With A = [[I, dt I], [0, I]], B = [[b1 I], [b2 I]] and the diagonal weights that
-// the problem has, every matrix of the Riccati recursion of Sec. IV.B couples a
-// position component with its own velocity only: P_t, K_t, S_t and P_{t+1}B fall apart into one two-state,
+// With A = [[I, dt I], [0, a22 I]], B = [[b1 I], [b2 I]] (the double integrator has
+// a22 = 1; HET: per-agent models, each with its own dt, a22, b1, b2) and the
+// diagonal weights that the problem has, every matrix of the Riccati recursion of
+// Sec. IV.B couples a position component with its own velocity only: P_t, K_t, S_t and P_{t+1}B fall apart into one two-state,
 // one-input recursion per axis, and the entries between axes are zeros.  The
 // general products form those zeros and add them; here they are left out, and
 // every other value is formed by the same operations in the same order, so the
@@ -20,6 +21,8 @@
 // 4096-scenario mixed batch over 500 iterations 769 -> 546 ms, a 512-agent 3D
 // swarm 2.76 -> 1.73 ms per iteration in graph mode, a two-agent crossing
 // 2.58 -> 1.49 ms; 1024 scenarios in float32 over 200 iterations 117 -> 69 ms.
+// Agents of unlike mass and damping, which took the dense products on one lane
+// each: 256 scenarios of 5 to 32 agents over 100 iterations 244 -> 55 ms.
 #pragma once
 
 namespace tadmm {
@@ -64,7 +67,7 @@ struct AxisView {
   const F* qf;      // rows of Qf, x_ref and x_init, shifted to axis c0
   const F* xr;
   const F* xi;
-  F rho, dt, b1, b2, lo[AX], hi[AX];
+  F rho, dt, a22, b1, b2, lo[AX], hi[AX];
   int N, T, ks, c0, nc;
 
   __device__ __forceinline__ F& C(int t, int w, int a) const { return cache[((t * AxisCache::E + w) * DP + a) * N]; }
@@ -80,6 +83,7 @@ struct AxisView {
 template <int AX, typename F, int NX, int NU, int DP>
 __device__ __forceinline__ void axis_model(AxisView<F, NX, NU, DP, AX>& V, const Model<F, NX, NU>& M) {
   V.dt = M.A[0][DP];
+  V.a22 = M.A[DP][DP];
   V.b1 = M.B[0][0];
   V.b2 = M.B[DP][0];
 #pragma unroll
@@ -148,7 +152,7 @@ __device__ __forceinline__ AxisView<F, NX, NU, DP, 1> axis_view_of(const AgentCt
 // AX == DP: the calling lane's own agent; `act` may differ between lanes.
 // AX == 1: lanes gb .. gb + DP - 1 hold the axes of one agent and exchange their S;
 // every lane of the warp calls this.  Returns 1 on a non-positive pivot.
-template <typename F, int NX, int NU, int DP, int AX>
+template <bool HET, typename F, int NX, int NU, int DP, int AX>
 __device__ __forceinline__ int axis_factor(const AxisView<F, NX, NU, DP, AX>& V, bool act, int dirty, int gb) {
   using AC = AgentConst<NX, NU>;
   using L = AxisCache;
@@ -184,8 +188,13 @@ __device__ __forceinline__ int axis_factor(const AxisView<F, NX, NU, DP, AX>& V,
 #pragma unroll
     for (int a = 0; a < AX; ++a) {
       // PA = [[pp, pav], [pv, pvv]], PB = [pb1; pb2]
-      pav[a] = fma(pp[a], V.dt, pv[a]);
-      pvv[a] = fma(pv[a], V.dt, vv[a]);
+      if constexpr (HET) {  // the order of the general products
+        pav[a] = fma(pv[a], V.a22, pp[a] * V.dt);
+        pvv[a] = fma(vv[a], V.a22, pv[a] * V.dt);
+      } else {
+        pav[a] = fma(pp[a], V.dt, pv[a]);
+        pvv[a] = fma(pv[a], V.dt, vv[a]);
+      }
       pb1[a] = fma(pv[a], V.b2, pp[a] * V.b1);
       pb2[a] = fma(vv[a], V.b2, pv[a] * V.b1);
       const bool hd = V.held(mask, a);
@@ -229,7 +238,7 @@ __device__ __forceinline__ int axis_factor(const AxisView<F, NX, NU, DP, AX>& V,
         // P_t = Qbar_t + A'(P A) + M'K
         const F npp = fma(mp[a], k1, V.k(AC::QB + a) + pp[a]);
         const F npv = fma(mp[a], k2, pav[a]);
-        const F nvv = fma(mv[a], k2, fma(V.dt, pav[a], V.k(AC::QB + DP + a)) + pvv[a]);
+        const F nvv = fma(mv[a], k2, fma(HET ? V.a22 : F(1), pvv[a], fma(V.dt, pav[a], V.k(AC::QB + DP + a))));
         pp[a] = npp;
         pv[a] = npv;
         vv[a] = nvv;
@@ -254,7 +263,7 @@ enum { PASS_OUT = 1, PASS_BAD = 2, PASS_MULT = 4, PASS_NAN = 8 };
 // inputs decide only where one is negative, so in float64 their sign is taken
 // from a float32 value with a margin over its error, and mult_scan forms them
 // where that leaves a doubt.
-template <typename F, int NX, int NU, int DP, int AX>
+template <bool HET, typename F, int NX, int NU, int DP, int AX>
 __device__ __forceinline__ int axis_pass(const AxisView<F, NX, NU, DP, AX>& V) {
   using AC = AgentConst<NX, NU>;
   using L = AxisCache;
@@ -308,8 +317,9 @@ __device__ __forceinline__ int axis_pass(const AxisView<F, NX, NU, DP, AX>& V) {
         const F e1 = fma(hd ? g1[a] : F(1), hd ? ub : qp, pn[a]);
         const F e2 = fma(hd ? F(1) : g1[a], hd ? qp : bp, e1);
         const F f1 = fma(hd ? g2[a] : V.dt, hd ? ub : pn[a], hd ? vn[a] : qv);
-        const F f2 = fma(hd ? V.dt : F(1), hd ? e1 : vn[a], hd ? qv : f1);
-        const F f3 = fma(hd ? F(1) : g2[a], hd ? f1 : bp, f2);
+        const F a22 = HET ? V.a22 : F(1);
+        const F f2 = fma(hd ? V.dt : a22, hd ? e1 : vn[a], hd ? qv : f1);
+        const F f3 = fma(hd ? a22 : g2[a], hd ? f1 : bp, f2);
         pn[a] = e2;
         vn[a] = f3;
       }
@@ -358,7 +368,7 @@ __device__ __forceinline__ int axis_pass(const AxisView<F, NX, NU, DP, AX>& V) {
       if (!hd && ((ku < kmin[a]) | (ku > kmax[a]))) found |= PASS_OUT;
       const F u = hd ? V.bound(mask, a) : uf;
       xp[a] = fma(V.b1, u, fma(V.dt, xv[a], xp[a]));
-      xv[a] = fma(V.b2, u, xv[a]);
+      xv[a] = fma(V.b2, u, HET ? V.a22 * xv[a] : xv[a]);
       if (hd) {
         // multiplier +-(Rbar u + B'lambda_{t+1}), B'lambda_{t+1} = (P_{t+1}B)'x_{t+1} + B'p_{t+1}
         const bool low = (mask >> (V.c0 + a)) & 1u;
@@ -395,9 +405,9 @@ __device__ __forceinline__ int axis_pass(const AxisView<F, NX, NU, DP, AX>& V) {
 // whatever the number of active lanes, so when the agents' axes fit the warp's
 // lanes they take one lane each, and otherwise each lane takes its own agent,
 // all axes.  Returns the pass's findings to the lane that owns the agent.
-template <typename F, int NX, int NU, int DP, bool PASS = true>
-__device__ __forceinline__ int axis_round(const AgentCtx<F, NX, NU, DP>& A, bool go, int dirty,
-                                          unsigned long long& nfact) {
+template <bool HET, bool PASS, typename F, int NX, int NU, int DP>
+__device__ __forceinline__ int axis_round_of(const AgentCtx<F, NX, NU, DP>& A, bool go, int dirty,
+                                             unsigned long long& nfact) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NG = 32 / DP;  // agents whose axes fit a warp
   const unsigned owners = __ballot_sync(FULL, go);
@@ -413,10 +423,10 @@ __device__ __forceinline__ int axis_round(const AgentCtx<F, NX, NU, DP>& A, bool
     const int src = act ? __ffs(m) - 1 : lane;
     const AxisView<F, NX, NU, DP, 1> V = axis_view_of<F, NX, NU, DP>(A, src, act ? lane - gb : 0);
     const int od = __shfl_sync(FULL, dirty, src);
-    if (axis_factor<F, NX, NU, DP, 1>(V, act, od, act ? gb : 0)) found = PASS_BAD;
+    if (axis_factor<HET>(V, act, od, act ? gb : 0)) found = PASS_BAD;
     __syncwarp();
     if constexpr (PASS) {
-      if (act) found |= axis_pass<F, NX, NU, DP, 1>(V);
+      if (act) found |= axis_pass<HET>(V);
       __syncwarp();
     }
     int all = 0;
@@ -426,11 +436,17 @@ __device__ __forceinline__ int axis_round(const AgentCtx<F, NX, NU, DP>& A, bool
     found = all;
   } else if (go) {
     const AxisView<F, NX, NU, DP, DP> V = axis_view<F, NX, NU, DP>(A);
-    if (axis_factor<F, NX, NU, DP, DP>(V, true, dirty, 0)) found = PASS_BAD;
-    if constexpr (PASS) found |= axis_pass<F, NX, NU, DP, DP>(V);
+    if (axis_factor<HET>(V, true, dirty, 0)) found = PASS_BAD;
+    if constexpr (PASS) found |= axis_pass<HET>(V);
   }
   __syncwarp();
   return go ? found : 0;
+}
+
+template <typename F, int NX, int NU, int DP, bool PASS = true>
+__device__ __forceinline__ int axis_round(const AgentCtx<F, NX, NU, DP>& A, bool go, int dirty,
+                                          unsigned long long& nfact) {
+  return A.het ? axis_round_of<true, PASS>(A, go, dirty, nfact) : axis_round_of<false, PASS>(A, go, dirty, nfact);
 }
 
 // Multipliers of the held inputs of the agents of the lanes with `need`: the

@@ -276,6 +276,7 @@ struct AgentCtx {
   const F* xi;
   int coop;          // one lane per axis allowed (uniform over the warp)
   int nc;            // consensus copies of the agent (its number of pairs)
+  int het;           // per-agent models (uniform over the batch)
 
   __device__ __forceinline__ F k(int e) const { return kc[e * ks]; }
 
@@ -995,7 +996,8 @@ __device__ __forceinline__ AgentCtx<F, NX, NU, DP> make_agent(const Dev<F>& D, c
                                                               int ks, double rho) {
   using AC = AgentConst<NX, NU>;
   AgentCtx<F, NX, NU, DP> A;
-  A.M = DI ? &M : &agent_model<F, NX, NU>(D, M, s, i);  // the structured path has one model
+  A.M = &agent_model<F, NX, NU>(D, M, s, i);
+  A.het = D.models != nullptr;
   A.N = s.N;
   A.T = s.T;
   A.i = i;
@@ -1029,7 +1031,7 @@ __device__ __forceinline__ AgentCtx<F, NX, NU, DP> make_agent(const Dev<F>& D, c
 
 // Context of a lane that owns no agent in this x-update (it only helps).
 template <typename F, int NX, int NU, int DP>
-__device__ __forceinline__ AgentCtx<F, NX, NU, DP> idle_agent(const Model<F, NX, NU>& M, F* kc, int ks, int coop) {
+__device__ __forceinline__ AgentCtx<F, NX, NU, DP> idle_agent(const Dev<F>& D, const Model<F, NX, NU>& M, F* kc, int ks) {
   AgentCtx<F, NX, NU, DP> A;
   A.M = &M;
   A.N = 1;
@@ -1047,8 +1049,9 @@ __device__ __forceinline__ AgentCtx<F, NX, NU, DP> idle_agent(const Model<F, NX,
   A.qf = nullptr;
   A.xr = nullptr;
   A.xi = nullptr;
-  A.coop = coop;
+  A.coop = D.coop;
   A.nc = 0;
+  A.het = D.models != nullptr;
   return A;
 }
 
@@ -1102,7 +1105,7 @@ __device__ int eqp_direction(const AgentCtx<F, NX, NU, DP>& A, const F* hprev, F
     // one axis after the other, on the axis words of the factor cache
     using L = AxisCache;
     const AxisView<F, NX, NU, DP, DP> V = axis_view<F, NX, NU, DP>(A);
-    const F a22 = Mo.A[DP][DP];  // 1, read so that the product below stays rounded
+    const F a22 = Mo.A[DP][DP];  // where it is 1, read so that the product below stays rounded
     int bad = 0;
     for (int a = 0; a < DP; ++a) {
       F pp = dq(T, a), pv = dq(T, DP + a);
@@ -1123,7 +1126,7 @@ __device__ int eqp_direction(const AgentCtx<F, NX, NU, DP>& A, const F* hprev, F
         const F g1 = V.C(t, L::G1, a), g2 = V.C(t, L::G2, a), k = V.C(t, L::D, a);
         const F u = hd ? F(0) : fma(g2, xv, fma(g1, xp, k));
         xp = fma(V.b1, u, fma(V.dt, xv, xp));
-        xv = fma(V.b2, u, xv);
+        xv = fma(V.b2, u, a22 * xv);
         A.us(t, a) = u;
         F d = F(0);
         if (hd) {
@@ -1370,7 +1373,7 @@ __device__ int xupdate_phase(const Dev<F>& D, const Model<F, NX, NU>& M, const S
     const bool has = r < mine;
     const AgentCtx<F, NX, NU, DP> A =
         has ? make_agent<F, NX, NU, DP, DI>(D, M, s, i0 + r * stride, lvl_out, kcs + threadIdx.x, blockDim.x, s.rho)
-            : idle_agent<F, NX, NU, DP>(M, kcs + threadIdx.x, blockDim.x, D.coop);
+            : idle_agent<F, NX, NU, DP>(D, M, kcs + threadIdx.x, blockDim.x);
     int res = ST_CONVERGED;
     if constexpr (HOMO) {
       // warp-collective: every lane enters when any lane's agent takes a
@@ -2174,7 +2177,7 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
       const ScenMeta& s = gs.meta[has ? my_m : 0];
       const AgentCtx<F, NX, NU, DP> A = has ? make_agent<F, NX, NU, DP, DI>(D, M, s, my_i, xl ^ 1, kcs + tid, nt,
                                                                         gs.rho[my_m])
-                                            : idle_agent<F, NX, NU, DP>(M, kcs + tid, nt, D.coop);
+                                            : idle_agent<F, NX, NU, DP>(D, M, kcs + tid, nt);
       const int as_max = D.as_max > 0 ? D.as_max : 10 * s.T * NU + 10;
       const F eps = D.eps_rel > 0 ? F(D.eps_rel) : (sizeof(F) == 8 ? F(1e-12) : F(1e-5));
       const int st = xupdate_agent<F, NX, NU, DP, DI>(A, has, start_kind_of(D, k), as_max, eps, neqp,

@@ -100,7 +100,8 @@ struct tadmm_handle {
 
   // batched mode launch shape and captured graph
   int tpc = 0, cps = 0, variant = 0;
-  int di = 0;               // model is an exact double integrator (structured kernel path)
+  int di = 0;               // the shared model is an exact double integrator
+  int ax = 0;               // it is, or every agent's own model is axis-separable (tadmm_axis.cuh)
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   double g_tol = -1.0;

@@ -704,7 +704,7 @@ int Impl<F, NX, NU, DP>::max_ctas_per_sm(int tpc, int variant, const tadmm_handl
   int n = 0;
   if (tpc > variant_maxt(variant)) return 0;
   const size_t smem = (h ? fused_smem_bytes<F, DP>(h, nullptr) : 0) + agent_const_bytes<F, NX, NU>(tpc);
-  const void* kfn = batched_kernel<F, NX, NU, DP>(variant, h ? h->di != 0 : false);
+  const void* kfn = batched_kernel<F, NX, NU, DP>(variant, h ? h->ax != 0 : false);
   // 48 KB without it, the static part (about 11 KB) included
   if (smem > 32 * 1024) cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kfn, tpc, smem) != cudaSuccess) {
@@ -747,7 +747,7 @@ int Impl<F, NX, NU, DP>::solve_batched(tadmm_handle* h, double tol, int max_iter
     if (rc) return rc;
     cudaMemsetAsync(h->queue, 0, sizeof(int32_t), h->cap_stream);
     void* args[] = {&D};
-    cudaLaunchKernel(batched_kernel<F, NX, NU, DP>(var, h->di != 0), dim3(grid), dim3(tpc), args, smem, h->cap_stream);
+    cudaLaunchKernel(batched_kernel<F, NX, NU, DP>(var, h->ax != 0), dim3(grid), dim3(tpc), args, smem, h->cap_stream);
     cudaError_t le = cudaGetLastError();
     cudaError_t ee = cudaStreamEndCapture(h->cap_stream, &g);
     if (le != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_check(le, "batched kernel launch"); }
@@ -801,7 +801,7 @@ int Impl<F, NX, NU, DP>::solve_plain(tadmm_handle* h, double tol, int max_iter, 
       const int tk = k % 3, tkp1 = (k + 1) % 3, tkm1 = (k + 2) % 3;
       cudaMemsetAsync(h->flag, 0, sizeof(int32_t), st);
       cudaMemsetAsync(h->red2, 0, 2 * sizeof(unsigned long long), st);
-      if (h->di)
+      if (h->ax)
         if (homo)
           k_xupdate<F, NX, NU, DP, true, true><<<(s.N + apw - 1) / apw, 32, 0, st>>>(D, sc, k, xl ^ 1, h->flag, apw);
         else
@@ -919,7 +919,7 @@ int Impl<F, NX, NU, DP>::solve_graph(tadmm_handle* h, double tol, int max_iter, 
     const dim3 gx((unsigned)((h->tot_agents + gapw - 1) / gapw));
     const dim3 gp(grid_for(h->tot_pairs, 128, 1 << 30), tmax);
     const dim3 gg(h->n_gblk, tmax);
-    if (h->di)
+    if (h->ax)
       if (homo)
         k_g_xupdate<F, NX, NU, DP, true, true><<<gx, 32, 0, h->cap_stream>>>(D, G, h->agent_scen, h->tot_agents, gapw);
       else

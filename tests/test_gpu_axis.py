@@ -4,7 +4,7 @@ the shortest horizons."""
 import numpy as np
 import pytest
 
-from instances import make_batch, random_scenario
+from instances import heterogeneous_agents, make_batch, random_scenario
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +59,32 @@ def test_large_magnitudes_and_held_multipliers():
         d, cd = _run(c, flags=tg.FLAG_NO_STRUCTURE)
         assert np.array_equal(g["W"], d["W"]) and np.array_equal(cg["eqp"], cd["eqp"])
         assert np.abs(g["X"] - d["X"]).max() <= 1e-12 * np.abs(d["X"]).max()
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("dp,N,T", [(2, 1, 3), (2, 16, 7), (2, 17, 7), (3, 11, 6)])
+def test_axis_recursions_per_agent_models(dp, N, T, precision):
+    """Agents of unlike mass and damping: the per-axis recursions give the bits of the
+    dense products, in both modes; and after an update to models that couple the
+    axes (and back) the handle takes the products that these need."""
+    import dataclasses
+
+    import paper_2602_15838_gb300 as tg
+    b = heterogeneous_agents(_one(dp, N, T, seed=31 + N), seed=4)
+    ref, cref = _run(b, precision=precision, flags=tg.FLAG_NO_STRUCTURE)
+    for kw in (dict(), dict(flags=tg.FLAG_NO_LANE_GROUPS), dict(mode="graph")):
+        g, c = _run(b, precision=precision, **kw)
+        for k in ("X", "U", "theta", "W", "status", "iters"):
+            assert np.array_equal(g[k], ref[k]), (kw, k)
+        assert np.array_equal(c["eqp"], cref["eqp"]), kw
+    A2 = b.A_agent.copy()
+    A2[:, 0, 1] = 0.01
+    mixed = dataclasses.replace(b, A_agent=A2)
+    want, _ = _run(mixed, precision=precision, flags=tg.FLAG_NO_STRUCTURE)
+    s = tg.Solver(b, precision=precision)
+    for data, exp in ((b, ref), (mixed, want), (b, ref)):
+        s.update(data)
+        s.solve(0.0, 9)
+        out = s.solution()
+        assert np.array_equal(out["X"], exp["X"]) and np.array_equal(out["W"], exp["W"])
+    s.close()
