@@ -51,6 +51,11 @@ __device__ __forceinline__ float near_f32(double v) {
   return __uint_as_float(r | (hi & 0x80000000u));
 }
 
+__device__ __forceinline__ float near_f32(float v) {
+  return fabsf(v) < 0x1p60f ? v : __uint_as_float(0x7FC00000u);
+}
+__device__ __forceinline__ float near_f32(df64 v) { return near_f32(v.hi); }
+
 // Part of an agent's data that a lane works on: AX axes from c0 on (all of them,
 // or one when the agents of a round are spread over lanes).  Pointers are those
 // of the agent's first axis; word w of an axis a lies a * N further on.
@@ -447,6 +452,122 @@ template <typename F, int NX, int NU, int DP, bool PASS = true>
 __device__ __forceinline__ int axis_round(const AgentCtx<F, NX, NU, DP>& A, bool go, int dirty,
                                           unsigned long long& nfact) {
   return A.het ? axis_round_of<true, PASS>(A, go, dirty, nfact) : axis_round_of<false, PASS>(A, go, dirty, nfact);
+}
+
+// Ratio test (see ratio_test) of the agents of the lanes with `need`, into o.  The
+// warp takes one agent at a time, its inputs spread over the lanes: 2 FP64
+// instructions per 32 inputs and 2 per candidate, where one lane per agent takes 4
+// per input of the warp's longest loop (8 per stage in 2D beside the 14 or 28 of a
+// pass).  The smallest ratio comes out of the same comparisons num aden < anum den
+// in index order as there, taken over the candidates alone: the inputs whose float32
+// ratio is within 2^-18 of the smallest one's.  Any other ratio is larger than that
+// by far more than the comparisons' rounding, so it can neither win nor stand in a
+// winner's way.  A 512-agent 3D swarm over its first 20 iterations: 34.9 -> 30.2 ms,
+// 200 small 3D swarms over 60: 64.4 -> 61.8 ms; the 4096-scenario batch, most of
+// whose rounds do not block, is level.  Every lane of the warp calls this.
+template <typename F, int NX, int NU, int DP>
+__device__ void ratio_scan(const AgentCtx<F, NX, NU, DP>& A, bool need, EqpScan<F>& o) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int kKeep = 4;  // inputs per lane that stay in registers between the two passes
+  const Model<F, NX, NU>& Mo = *A.M;
+  const int lane = threadIdx.x & 31;
+  for (unsigned rem = __ballot_sync(FULL, need); rem; rem &= rem - 1) {
+    const int src = __ffs(rem) - 1;
+    auto sp = [&](auto p) { return (decltype(p))__shfl_sync(FULL, (unsigned long long)p, src); };
+    const uint16_t* const Wm = sp(A.Wm);
+    const F* const U = sp(A.U);
+    const F* const Us = sp(A.Us);
+    const int N = __shfl_sync(FULL, A.N, src), n = __shfl_sync(FULL, A.T, src) * NU;
+    const int i = __shfl_sync(FULL, A.i, src);
+    // distance to the bound (at least 0) and size of the step of input e; false if it cannot block
+    auto ratio = [&](int e, F& num, F& den, bool& lower) -> bool {
+      const int t = e / NU, a = e - t * NU;
+      if (e >= n || ((Wm[t * N + i] >> a) & 0x101u)) return false;
+      const F cu = U[e * N + i], p = Us[e * N + i] - cu;
+      const unsigned long long pb = abs_bits(p);
+      if (pb == ord_bits(F(0))) return false;
+      lower = sign_set(p);
+      const F lo = a == 0 ? Mo.umin[0] : (a == 1 ? Mo.umin[1] : Mo.umin[NU - 1]);
+      const F hi = a == 0 ? Mo.umax[0] : (a == 1 ? Mo.umax[1] : Mo.umax[NU - 1]);
+      num = (lower ? cu : hi) - (lower ? lo : cu);
+      if (sign_set(num)) num = F(0);
+      den = from_bits(pb, F(0));
+      return true;
+    };
+    // float32 bounds of the ratio: both operands cut to 24 bits (2^-23 each), one division
+    auto low_of = [&](F num, F den, float& up) -> float {
+      const float r = near_f32(num) / near_f32(den);
+      up = r < 1e-30f ? 1e-30f : r * (1.0f + 0x1p-19f);
+      return r < 1e-30f ? 0.0f : r * (1.0f - 0x1p-19f);
+    };
+    F num[kKeep], den[kKeep];
+    float low[kKeep];
+    bool neg[kKeep], has[kKeep];
+    float lim = 1.0f;
+    for (int e0 = 0; e0 < n; e0 += 32 * kKeep) {
+#pragma unroll
+      for (int j = 0; j < kKeep; ++j) {
+        has[j] = ratio(e0 + 32 * j + lane, num[j], den[j], neg[j]);
+        float up = 1.0f;
+        low[j] = has[j] ? low_of(num[j], den[j], up) : 0.0f;
+        if (has[j] && up < lim) lim = up;
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) lim = fminf(lim, __shfl_xor_sync(FULL, lim, off));
+    F anum = F(1), aden = F(1);
+    int blk = -1, side = 0;
+    for (int e0 = 0; e0 < n; e0 += 32 * kKeep) {
+#pragma unroll
+      for (int j = 0; j < kKeep; ++j) {
+        if (n > 32 * kKeep) {
+          has[j] = ratio(e0 + 32 * j + lane, num[j], den[j], neg[j]);
+          float up;
+          low[j] = has[j] ? low_of(num[j], den[j], up) : 0.0f;
+        }
+        unsigned cand = __ballot_sync(FULL, has[j] && !(low[j] > lim));
+        const unsigned down = __ballot_sync(FULL, neg[j]);
+        for (; cand; cand &= cand - 1) {
+          const int l = __ffs(cand) - 1;
+          const F cn = shfl_f(num[j], l), cd = shfl_f(den[j], l);
+          if (mono_key(cn * aden) < mono_key(anum * cd)) {
+            anum = cn;
+            aden = cd;
+            blk = e0 + 32 * j + l;
+            side = (down >> l) & 1u ? 1 : 2;
+          }
+        }
+      }
+    }
+    if (lane == src) {
+      o.anum = anum;
+      o.aden = aden;
+      o.blk = blk;
+      o.bside = side;
+    }
+  }
+}
+
+// u <- u + alpha (us - u) for the agents of the lanes with `need`, the warp taking
+// one agent at a time.  Every lane of the warp calls this.
+template <typename F, int NX, int NU, int DP>
+__device__ void step_scan(const AgentCtx<F, NX, NU, DP>& A, bool need, F alpha) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  for (unsigned rem = __ballot_sync(FULL, need); rem; rem &= rem - 1) {
+    const int src = __ffs(rem) - 1;
+    auto sp = [&](auto p) { return (decltype(p))__shfl_sync(FULL, (unsigned long long)p, src); };
+    F* const U = sp(A.U);
+    const F* const Us = sp(A.Us);
+    const int N = __shfl_sync(FULL, A.N, src), n = __shfl_sync(FULL, A.T, src) * NU;
+    const int i = __shfl_sync(FULL, A.i, src);
+    const F al = shfl_f(alpha, src);
+    for (int e = lane; e < n; e += 32) {
+      const F cu = U[e * N + i];
+      U[e * N + i] = fma(al, Us[e * N + i] - cu, cu);
+    }
+  }
+  __syncwarp();
 }
 
 // Multipliers of the held inputs of the agents of the lanes with `need`: the

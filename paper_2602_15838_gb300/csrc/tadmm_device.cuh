@@ -897,10 +897,14 @@ __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int sta
       o.anum = 1; o.aden = 1; o.blk = -1; o.bside = 0; o.worst = 0; o.widx = -1; o.scale = 1; o.bad = 0;
       bad = found & PASS_BAD;
       // the multipliers count only when nothing blocks the step
-      if (go && !bad && (found & PASS_OUT)) ratio_test<F, NX, NU, DP>(A, o);
+      ratio_scan<F, NX, NU, DP>(A, go && !bad && (found & PASS_OUT), o);
       const bool scan = go && !bad && (found & PASS_MULT) && (o.blk < 0 || (found & PASS_NAN));
       mult_scan<F, NX, NU, DP>(A, scan, o);
       o.out = 0;
+      // step to the blocking input's bound (nowhere when it sits there already)
+      const bool cut = go && !bad && !o.bad && o.blk >= 0;
+      const F alpha = cut ? o.anum / o.aden : F(0);
+      step_scan<F, NX, NU, DP>(A, cut && alpha != F(0), alpha);
     } else {
       refactor_sweep<F, NX, NU, DP>(A, go, dirty, nfact, bad);
       if (go) o = eqp_solve<F, NX, NU, DP>(A);
@@ -914,8 +918,10 @@ __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int sta
         dirty = -1;
         if (!DI && o.out) ratio_test<F, NX, NU, DP>(A, o);
         if (o.blk >= 0) {
-          const F alpha = o.anum / o.aden;
-          step_inputs<F, NX, NU, DP>(A, T, false, alpha);
+          if constexpr (!DI) {
+            const F alpha = o.anum / o.aden;
+            step_inputs<F, NX, NU, DP>(A, T, false, alpha);
+          }
           const int bt = o.blk / NU, ba = o.blk - bt * NU;
           A.u(bt, ba) = (o.bside == 1) ? Mo.umin[ba] : Mo.umax[ba];
           A.W(bt) = (uint16_t)(A.W(bt) | (o.bside == 1 ? (1u << ba) : (0x100u << ba)));

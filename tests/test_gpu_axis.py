@@ -88,3 +88,21 @@ def test_axis_recursions_per_agent_models(dp, N, T, precision):
         out = s.solution()
         assert np.array_equal(out["X"], exp["X"]) and np.array_equal(out["W"], exp["W"])
     s.close()
+
+
+@pytest.mark.parametrize("dp,N,T", [(2, 3, 16), (2, 5, 33), (3, 4, 22), (2, 2, 70), (3, 18, 5)])
+@pytest.mark.parametrize("start", ["turbo", "cold"])
+def test_ratio_test_over_the_lanes(dp, N, T, start):
+    """The ratio test that spreads an agent's inputs over the lanes (32 and 64 of
+    them are the edges of what it keeps in registers) blocks on the same inputs as
+    the general code's test in index order: the same counts and working sets on
+    tight boxes, where most rounds block."""
+    import paper_2602_15838_gb300 as tg
+    b = random_scenario(seed=11 * N + T, N=N, T=T, dp=dp, box=6.0, umax=0.15)
+    g, cg = _run(b, start=start)
+    d, cd = _run(b, start=start, flags=tg.FLAG_NO_STRUCTURE)
+    assert np.array_equal(cg["eqp"], cd["eqp"]) and np.array_equal(g["W"], d["W"])
+    for k in ("X", "U", "theta"):
+        assert np.abs(d[k] - g[k]).max(initial=0.0) <= 1e-11 * max(1.0, np.abs(d[k]).max(initial=0.0)), k
+    h, ch = _run(b, start=start, mode="graph")
+    assert np.array_equal(h["X"], g["X"]) and np.array_equal(ch["eqp"], cg["eqp"])
