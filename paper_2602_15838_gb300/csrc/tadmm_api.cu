@@ -229,7 +229,7 @@ static void free_all(tadmm_handle* h) {
   if (!h) return;
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->wexec) cudaGraphExecDestroy(h->wexec);
-  void* gptrs[] = {h->gs_iter, h->gs_active, h->gs_need, h->gs_fail, h->gs_rb, h->gs_sb, h->gs_blk};
+  void* gptrs[] = {h->gs_iter, h->gs_active, h->gs_fail, h->gs_rb, h->gs_sb, h->gs_on, h->gs_done, h->gs_blk};
   for (void* p : gptrs)
     if (p) cudaFree(p);
   void* ptrs0[] = {h->goff, h->gmem, h->gorder};
@@ -392,6 +392,8 @@ extern "C" int tadmm_create(const tadmm_batch* b, const tadmm_options* opt, tadm
     m.ps_off = h->tot_ps;
     m.xs_off = h->tot_xs;
     m.pair_off = h->tot_pairs;
+    m.on_off = h->tot_on;
+    if (!m.sparse) h->tot_on += (int64_t)m.T * ((m.N + 31) / 32) * m.N;
     m.d = b->d_min[s];
     m.rho = b->rho[s];
     h->tot_agents += m.N;

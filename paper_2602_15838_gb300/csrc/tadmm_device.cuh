@@ -48,6 +48,7 @@ struct ScenMeta {
   int64_t ps_off;     // pair-step offset (sum of P*T)
   int64_t xs_off;     // agent-state offset (sum of N*(T+1))
   int64_t pair_off;   // pair offset (sum of P)
+  int64_t on_off;     // word offset of the graph mode's partner masks (sum of T ceil(N / 32) N)
   double d, rho;
 };
 
@@ -1507,6 +1508,105 @@ __device__ void gather_phase(const Dev<F>& D, const ScenMeta& s, int xl_new, int
 #pragma unroll
     for (int c = 0; c < DP; ++c) h[((size_t)tm1 * DP + c) * N + i] = acc[c];
   }
+}
+
+// Whether pair-step q (agents i, j at step tm1 + 1) may move its projection step
+// away from zero: false where theta^k = 0 and the halfspace holds, so that
+// theta^{k+1} = 0 and the pair adds nothing to a residual or a sum.  In float64 from
+// a float32 value with a margin over its error (as in group_sweep), otherwise true.
+template <typename F, int DP>
+__device__ __forceinline__ bool pair_pushes(F th, F d, const F (&av)[DP], const F (&pi)[DP], const F (&pj)[DP]) {
+  if constexpr (!std::is_same<F, double>::value) return true;
+  float g = near_f32(d), size = fabsf(g);
+#pragma unroll
+  for (int c = 0; c < DP; ++c) {
+    const float af = near_f32(av[c]), fi = near_f32(pi[c]), fj = near_f32(pj[c]);
+    g = fmaf(-af, fi - fj, g);
+    size = fmaf(fabsf(af), fabsf(fi) + fabsf(fj), size);
+  }
+  return !(th == F(0) && g < -fmaf(size, 0x1p-19f, 1e-17f));
+}
+
+// pair_phase of one pair-step, leaving out the pairs that do not push; the others
+// enter themselves in their agents' partner masks `on` ([T][ceil(N / 32)][N] words,
+// nullptr for listed pairs).
+template <typename F, int NX, int DP>
+__device__ __forceinline__ void pair_step(const Dev<F>& D, const ScenMeta& s, int xl, int tk, int tkp1, int tm1, int pair,
+                                          uint32_t* on, unsigned long long& rb) {
+  const int N = s.N, P = s.P;
+  const F* Xn = D.X + (size_t)(xl ^ 1) * D.tot_xs * NX + s.xs_off * NX;
+  const F* a = D.a + s.ps_off * DP;
+  const int64_t q = s.ps_off + (int64_t)tm1 * P + pair;
+  const int pk = D.pairs[s.pair_off + pair], i = pk & 0xFFFF, j = pk >> 16;
+  const F th = D.theta[(size_t)tk * D.tot_ps + q];
+  F av[DP], pi[DP], pj[DP];
+#pragma unroll
+  for (int c = 0; c < DP; ++c) {
+    av[c] = a[((size_t)tm1 * DP + c) * P + pair];
+    const size_t ro = ((size_t)(tm1 + 1) * NX + c) * N;
+    pi[c] = Xn[ro + i];
+    pj[c] = Xn[ro + j];
+  }
+  F tn = F(0);
+  if (pair_pushes<F, DP>(th, F(s.d), av, pi, pj)) {
+    F g = F(s.d);  // d - a'(p_i - p_j)
+    unsigned long long amax = 0;
+#pragma unroll
+    for (int c = 0; c < DP; ++c) {
+      g = fma(-av[c], pi[c] - pj[c], g);
+      const unsigned long long ab = abs_bits(av[c]);
+      amax = ab > amax ? ab : amax;
+    }
+    tn = fma(g, F(0.5), th);
+    if (sign_set(tn)) tn = F(0);
+    const unsigned long long v = abs_bits((tn - th) * from_bits(amax, F(0)));
+    rb = v > rb ? v : rb;
+    if (on && (tn != F(0) || th != F(0))) {
+      const int W = (N + 31) >> 5;
+      atomicOr(&on[((size_t)tm1 * W + (j >> 5)) * N + i], 1u << (j & 31));
+      atomicOr(&on[((size_t)tm1 * W + (i >> 5)) * N + j], 1u << (i & 31));
+    }
+  }
+  D.theta[(size_t)tkp1 * D.tot_ps + q] = tn;
+}
+
+// gather_phase of agent i at step tm1 over the partners in its mask, which it
+// clears (listed pairs: over its list).
+template <typename F, int NX, int NU, int DP>
+__device__ __forceinline__ void gather_step(const Dev<F>& D, const ScenMeta& s, int xl_new, int tkp1, int tk, int tm1,
+                                            int i, uint32_t* on) {
+  const int N = s.N, P = s.P;
+  const F* Xn = D.X + (size_t)xl_new * D.tot_xs * NX + s.xs_off * NX;
+  const F* thn = D.theta + (size_t)tkp1 * D.tot_ps + s.ps_off + (size_t)tm1 * P;
+  const F* tho = D.theta + (size_t)tk * D.tot_ps + s.ps_off + (size_t)tm1 * P;
+  const F* a = D.a + s.ps_off * DP + (size_t)tm1 * DP * P;
+  const F nc = F(agent_nc(D, s, i));
+  F acc[DP];
+#pragma unroll
+  for (int c = 0; c < DP; ++c) acc[c] = nc * Xn[((size_t)(tm1 + 1) * NX + c) * N + i];
+  auto add = [&](int pair, bool first) {
+    F e = fma(F(2), thn[pair], -tho[pair]);
+    if (!first) e = -e;
+#pragma unroll
+    for (int c = 0; c < DP; ++c) acc[c] = fma(e, a[(size_t)c * P + pair], acc[c]);
+  };
+  if (s.sparse) {
+    for_partners(D, s, i, add);
+  } else {
+    const int W = (N + 31) >> 5;
+    for (int w = 0; w < W; ++w) {
+      uint32_t* const word = &on[((size_t)tm1 * W + w) * N + i];
+      uint32_t m = *word;
+      if (m) *word = 0;
+      for (; m; m &= m - 1) {
+        const int j = w * 32 + __ffs(m) - 1;
+        add(i < j ? pair_index(N, i, j) : pair_index(N, j, i), i < j);
+      }
+    }
+  }
+  F* h = D.h + s.as_off * DP;
+#pragma unroll
+  for (int c = 0; c < DP; ++c) h[((size_t)tm1 * DP + c) * N + i] = acc[c];
 }
 
 // Shared-memory tile of the tiled gather: for 32 own agents (rows) x 32

@@ -26,6 +26,7 @@ struct BwdBufs {
 
 struct tadmm_handle {
   int prec = 64, nx = 0, nu = 0, dp = 0, n_scen = 0;
+  int64_t tot_on = 0;       // words of the graph mode's partner masks
   int64_t tot_agents = 0, tot_as = 0, tot_ps = 0, tot_xs = 0, tot_pairs = 0;
   tadmm_options opt{};
   std::vector<int32_t> N, T;
@@ -112,8 +113,8 @@ struct tadmm_handle {
   BwdBufs bwd;
 
   // graph mode (conditional WHILE node over the per-iteration phase kernels)
-  void *gs_iter = nullptr, *gs_active = nullptr, *gs_need = nullptr, *gs_fail = nullptr, *gs_rb = nullptr,
-       *gs_sb = nullptr;
+  void *gs_iter = nullptr, *gs_active = nullptr, *gs_fail = nullptr, *gs_rb = nullptr,
+       *gs_sb = nullptr, *gs_on = nullptr, *gs_done = nullptr;
   void* gs_blk = nullptr;   // int2 (scenario, first agent) per 32-agent gather block
   int n_gblk = 0;
   cudaGraphExec_t wexec = nullptr;
