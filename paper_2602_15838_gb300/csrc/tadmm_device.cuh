@@ -815,10 +815,12 @@ __device__ __forceinline__ void step_inputs(const AgentCtx<F, NX, NU, DP>& A, in
 // an EQP solve takes it in the same pass, since a pass costs the warp the same
 // whatever number of lanes it serves.  Each lane's own sequence of working
 // sets, steps and multiplier tests is unchanged.
+// known_dirty: the last stage whose cached factors do not match the working set
+// (-1: none), or -2 to find it.
 // Returns ST_CONVERGED, ST_QP_FAIL or ST_NUMERIC.
 template <typename F, int NX, int NU, int DP, bool DI>
 __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int start_kind, int as_max, F eps_rel,
-                             unsigned long long& neqp, unsigned long long& nfact) {
+                             int known_dirty, unsigned long long& neqp, unsigned long long& nfact) {
   constexpr unsigned FULL = 0xffffffffu;
   const int T = has ? A.T : 0;
   const Model<F, NX, NU>& Mo = *A.M;
@@ -840,7 +842,8 @@ __device__ int xupdate_agent(const AgentCtx<F, NX, NU, DP>& A, bool has, int sta
       for (int t = 0; t < T; ++t) A.W(t) = 0;
     }
     // stages whose cached factors do not match the working set
-    for (int t0 = 0; t0 < T; t0 += kStageBatch) {
+    dirty = max(known_dirty, -1);
+    for (int t0 = 0; known_dirty < -1 && t0 < T; t0 += kStageBatch) {
       uint16_t cm[kStageBatch], w[kStageBatch];
 #pragma unroll
       for (int j = 0; j < kStageBatch; ++j) {
@@ -1390,8 +1393,10 @@ __device__ int xupdate_phase(const Dev<F>& D, const Model<F, NX, NU>& M, const S
         res = homotopy_agent<F, NX, NU, DP, DI>(A, hh, D.hprev + s.as_off * DP, D.mu + s.as_off * NU,
                                                D.dmu + s.as_off * NU, as_max, neqp, nfact);
     }
-    const int r2 = xupdate_agent<F, NX, NU, DP, DI>(A, has && res == ST_CONVERGED, kind, as_max, eps,
-                                                             neqp, nfact);
+    // a hot start finds its factors up to date, the first iteration finds none
+    const int known = HOMO ? -2 : (kind == QP_GIVEN ? -1 : (k == 0 ? s.T - 1 : -2));
+    const int r2 = xupdate_agent<F, NX, NU, DP, DI>(A, has && res == ST_CONVERGED, kind, as_max, eps, known, neqp,
+                                                    nfact);
     if (res == ST_CONVERGED) res = r2;
     if constexpr (HOMO) {
       if (has && res == ST_CONVERGED) homotopy_store<F, NX, NU, DP>(A, D.hprev + s.as_off * DP, D.mu + s.as_off * NU);
@@ -2269,6 +2274,7 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
   const int my_a = slot < nA ? slot : -1;  // in the group
   const int my_m = my_a >= 0 ? member_of(gs.aoff, G, my_a) : -1;
   const int my_i = my_a >= 0 ? my_a - gs.aoff[my_m] : 0;
+  bool stale = true;  // none of the agent's cached factors matches
   unsigned long long neqp = 0, nfact = 0;
   F* smE = sm;
   F* smA = sm + nP;
@@ -2286,8 +2292,10 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
                                             : idle_agent<F, NX, NU, DP>(D, M, kcs + tid, nt);
       const int as_max = D.as_max > 0 ? D.as_max : 10 * s.T * NU + 10;
       const F eps = D.eps_rel > 0 ? F(D.eps_rel) : (sizeof(F) == 8 ? F(1e-12) : F(1e-5));
-      const int st = xupdate_agent<F, NX, NU, DP, DI>(A, has, start_kind_of(D, k), as_max, eps, neqp,
-                                                                nfact);
+      const int kind = start_kind_of(D, k);
+      const int known = stale ? T - 1 : (kind == QP_GIVEN ? -1 : -2);
+      const int st = xupdate_agent<F, NX, NU, DP, DI>(A, has, kind, as_max, eps, known, neqp, nfact);
+      stale = false;
       if (has && st) atomicMax(&gs.flag[my_m], st);
     }
     __syncthreads();
@@ -2450,6 +2458,7 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
       if (my_m >= 0 && gs.adapt[my_m]) {
         const ScenMeta& s = gs.meta[my_m];
         for (int t = 0; t < s.T; ++t) D.Cm[s.as_off + (size_t)t * s.N + my_i] = 0xFFFF;
+        stale = true;
       }
       __syncthreads();
       if (tid < G) gs.adapt[tid] = 0;
