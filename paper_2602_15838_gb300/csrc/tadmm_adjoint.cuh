@@ -81,32 +81,42 @@ __global__ void k_bwd_init(Dev<F> D, BwdDev<F> B) {
   for (int64_t e = threadIdx.x; e < NT; e += blockDim.x) B.Wb[s.as_off + e] = D.Wm[s.as_off + e];
 }
 
-// Ordered compaction of the active halfspaces of one scenario (one warp).
+constexpr int kBwdThreads = 256;  // threads of a scenario's CTA here
+
+// Ordered compaction of the active halfspaces of one scenario (one CTA).
 template <typename F, int NX, int NU, int DP>
-__global__ void k_bwd_count(Dev<F> D, BwdDev<F> B) {
-  const int sc = blockIdx.x;
+__global__ void __launch_bounds__(kBwdThreads) k_bwd_count(Dev<F> D, BwdDev<F> B) {
+  constexpr int NW = kBwdThreads / 32;
+  __shared__ int part[NW];
+  const int sc = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const ScenMeta s = D.meta[sc];
-  const int lane = threadIdx.x;
   const uint8_t* hm = B.hmask + s.ps_off;
-  for (int i = lane; i < s.N; i += 32) B.amask[s.agent_off + i] = 0ull;
-  __syncwarp();
+  for (int i = tid; i < s.N; i += kBwdThreads) B.amask[s.agent_off + i] = 0ull;
+  __syncthreads();
   const int64_t PT = (int64_t)s.P * s.T;
   int count = 0;
-  for (int64_t base = 0; base < PT; base += 32) {
-    const int64_t q = base + lane;
+  for (int64_t base = 0; base < PT; base += kBwdThreads) {
+    const int64_t q = base + tid;
     const bool on = q < PT && hm[q] != 0;
     const unsigned ball = __ballot_sync(0xffffffffu, on);
+    if (lane == 0) part[w] = __popc(ball);
+    __syncthreads();
+    int pos = count + __popc(ball & ((1u << lane) - 1u));
+#pragma unroll
+    for (int v = 0; v < NW; ++v) {
+      if (v < w) pos += part[v];
+      count += part[v];
+    }
     if (on) {
-      const int pos = count + __popc(ball & ((1u << lane) - 1u));
       B.act[s.ps_off + pos] = (int32_t)q;
       const int tm1 = (int)(q / s.P), pair = (int)(q - (int64_t)tm1 * s.P);
       const int pk = D.pairs[s.pair_off + pair];
       atomicOr(&B.amask[s.agent_off + (pk & 0xFFFF)], 1ull << tm1);
       atomicOr(&B.amask[s.agent_off + (pk >> 16)], 1ull << tm1);
     }
-    count += __popc(ball);
+    __syncthreads();
   }
-  if (lane == 0) B.act_cnt[sc] = count;
+  if (tid == 0) B.act_cnt[sc] = count;
 }
 
 // Riccati solve of one agent's equality-constrained LQ problem with the cached
@@ -215,176 +225,333 @@ __device__ void lq_solve(const Model<F, NX, NU>& Mo, const F* cache, const uint1
   }
 }
 
-// In-place Cholesky S = L L' of an m x m SPD matrix in global memory by one
-// CTA (right-looking, lower triangle).  Returns 0, or 1 on a non-positive pivot.
-template <typename F>
-__device__ int cta_cholesky(F* S, int m, int* s_bad) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int k = 0; k < m; ++k) {
-    __syncthreads();
-    if (tid == 0) {
-      const F dkk = S[(size_t)k * m + k];
-      if (!(dkk > F(0))) *s_bad = 1;
-      S[(size_t)k * m + k] = sqrt_(dkk > F(0) ? dkk : F(1));
+// lq_solve for one axis of the double integrator, on the axis words of the factor
+// cache (tadmm_axis.cuh): the same values without the zeros between the axes.
+// The linear term starts at step tl (it is zero after it).  kk(t) is a word of
+// scratch per stage; outx(t, position, velocity), outu(t, u).
+template <typename F, int NX, int NU, class Lin, class Kk, class OutX, class OutU>
+__device__ __forceinline__ void lq_axis(const Model<F, NX, NU>& Mo, const F* cache, const uint16_t* Wm, int N, int i,
+                                        int T, int c, int tl, Lin lin, F xp, F xv, bool at_bounds, Kk kk, OutX outx,
+                                        OutU outu) {
+  using L = AxisCache;
+  constexpr int DP = NU;
+  // a11 = 1, read so that a product in the linear term stays rounded
+  const F a11 = Mo.A[0][0], dt = Mo.A[0][DP], b1 = Mo.B[0][0], b2 = Mo.B[DP][0];
+  auto C = [&](int t, int w) -> F { return cache[((size_t)(t * L::E + w) * DP + c) * N + i]; };
+  const std::true_type pos{};   // compile-time, so that a term of the positions only joins their product
+  const std::false_type vel{};
+  F pp = lin(tl, c, pos), pv = lin(tl, DP + c, vel);
+  for (int t = tl - 1; t >= 0; --t) {
+    const uint32_t mask = Wm[(size_t)t * N + i];
+    const bool hd = (mask >> c) & 0x101u;
+    F qp = pp, qv = pv;  // P_{t+1} B u_held + p_{t+1}
+    if (hd && at_bounds) {
+      const F ub = ((mask >> c) & 1u) ? Mo.umin[c] : Mo.umax[c], cp = b1 * ub, cv = b2 * ub;
+      qp = fma(C(t + 1, L::PV), cv, fma(C(t + 1, L::PP), cp, qp));
+      qv = fma(C(t + 1, L::VV), cv, fma(C(t + 1, L::PV), cp, qv));
     }
-    __syncthreads();
-    const F lkk = S[(size_t)k * m + k];
-    for (int r = k + 1 + tid; r < m; r += nt) S[(size_t)r * m + k] /= lkk;
-    __syncthreads();
-    const int rem = m - k - 1;
-    for (int e = tid; e < rem * rem; e += nt) {
-      const int r = k + 1 + e / rem, c = k + 1 + e % rem;
-      if (c <= r) S[(size_t)r * m + c] = fma(-S[(size_t)r * m + k], S[(size_t)c * m + k], S[(size_t)r * m + c]);
+    const F sv = hd ? F(0) : fma(b2, qv, b1 * qp);
+    kk(t) = -(C(t, L::SI) * sv);
+    if (t >= 1) {
+      pp = fma(a11, qp, lin(t, c, pos));
+      pv = fma(a11, qv, fma(dt, qp, lin(t, DP + c, vel)));
+      if (!hd) {
+        pp = fma(C(t, L::G1), sv, pp);
+        pv = fma(C(t, L::G2), sv, pv);
+      }
     }
   }
-  __syncthreads();
-  return *s_bad;
+  outx(0, xp, xv);
+  for (int t = 0; t < T; ++t) {
+    const uint32_t mask = Wm[(size_t)t * N + i];
+    F u = F(0);
+    if (!((mask >> c) & 0x101u)) u = fma(C(t, L::G2), xv, fma(C(t, L::G1), xp, t < tl ? F(kk(t)) : F(0)));
+    else if (at_bounds) u = ((mask >> c) & 1u) ? Mo.umin[c] : Mo.umax[c];
+    xp = fma(b1, u, fma(dt, xv, xp));
+    xv = fma(b2, u, xv);
+    outu(t, u);
+    outx(t + 1, xp, xv);
+  }
 }
 
-// x = S^{-1} b with the Cholesky factor of cta_cholesky (one thread).
+// Largest value of the CTA and the lowest index it has (kBwdThreads threads).
 template <typename F>
-__device__ void chol_solve_serial(const F* L, int m, F* x) {
-  for (int r = 0; r < m; ++r) {
-    F v = x[r];
-    for (int k = 0; k < r; ++k) v = fma(-L[(size_t)r * m + k], x[k], v);
-    x[r] = v / L[(size_t)r * m + r];
+__device__ __forceinline__ void cta_argmax(F& v, int& i, F* red_v, int* red_i) {
+  constexpr unsigned FULL = 0xffffffffu;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const F v2 = shfl_f(v, (threadIdx.x & 31) ^ o);
+    const int i2 = __shfl_xor_sync(FULL, i, o);
+    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
   }
-  for (int r = m - 1; r >= 0; --r) {
-    F v = x[r];
-    for (int k = r + 1; k < m; ++k) v = fma(-L[(size_t)k * m + r], x[k], v);
-    x[r] = v / L[(size_t)r * m + r];
+  if ((threadIdx.x & 31) == 0) {
+    red_v[threadIdx.x >> 5] = v;
+    red_i[threadIdx.x >> 5] = i;
   }
+  __syncthreads();
+  v = red_v[0];
+  i = red_i[0];
+#pragma unroll
+  for (int w = 1; w < kBwdThreads / 32; ++w) {
+    const F v2 = red_v[w];
+    const int i2 = red_i[w];
+    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
+  }
+  __syncthreads();
 }
+
+// The dense algebra below keeps, for every entry, the operations and the order
+// of the plain definitions (right-looking updates in step order, row sums in
+// column order) and changes only who does them and from where they read.  One
+// CTA works on a scenario's matrix of a few hundred rows, which is in L2 but not
+// in L1, so what bounds the plain forms is the latency of one dependent load per
+// multiplication: they are left-looking here, each thread with one row whose
+// entries of a step's column it sums up from consecutive words.
+// With the solves by axis below: 12 polishing rounds and a backward pass over 64
+// scenarios of 16 agents 72.9 -> 38.2 ms, 4 rounds over 9 scenarios of 20 agents
+// (several hundred rows) 489 -> 108 ms.  What is left is mostly warp_backward's
+// chain, m^2 / 2 multiply-adds of 68 cycles.
 
 // Rank-revealing Cholesky of the positive semidefinite m x m matrix S (full
 // symmetric storage) by one CTA, with diagonal pivoting: step k takes the
 // largest remaining diagonal entry (ties to the lowest position) and stops
 // when it is not above rank_tol times the largest diagonal entry of S.  The
-// pivot order goes to piv; afterwards L[r][c] = S[piv[r] m + piv[c]] for
-// r >= c, c < rank is the factor of the permuted matrix restricted to its
-// first `rank` columns ([L11; L21]).  Returns the rank (same in every thread).
+// pivot order goes to piv; column c of the factor replaces row piv[c] of S, by
+// the rows' own numbers.  d [m]: scratch.  Returns the rank (same in every thread).
 template <typename F>
-__device__ int cta_pivoted_cholesky(F* S, int m, int* piv, F rank_tol) {
-  __shared__ F red_v[128];
-  __shared__ int red_i[128];
-  __shared__ F s_dref;
-  __shared__ int s_stop;
+__device__ int cta_pivoted_cholesky(F* S, int m, int* piv, F* d, F rank_tol) {
+  __shared__ F red_v[kBwdThreads / 32];
+  __shared__ int red_i[kBwdThreads / 32];
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int r = tid; r < m; r += nt) piv[r] = r;
-  int rank = m;
-  for (int k = 0; k < m; ++k) {
-    __syncthreads();
-    F bv = F(-1);
-    int bi = m;
-    for (int j = k + tid; j < m; j += nt) {
-      const F v = S[(size_t)piv[j] * m + piv[j]];
-      if (v > bv) { bv = v; bi = j; }
-    }
-    red_v[tid] = bv;
-    red_i[tid] = bi;
-    __syncthreads();
-    for (int w = nt / 2; w > 0; w >>= 1) {
-      if (tid < w) {
-        const F v2 = red_v[tid + w];
-        const int i2 = red_i[tid + w];
-        if (v2 > red_v[tid] || (v2 == red_v[tid] && i2 < red_i[tid])) {
-          red_v[tid] = v2;
-          red_i[tid] = i2;
-        }
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      const F v = red_v[0];
-      const int j = red_i[0];
-      if (k == 0) s_dref = v;
-      if (j >= m || !(v > rank_tol * s_dref)) {
-        s_stop = 1;
-      } else {
-        s_stop = 0;
-        const int t = piv[k];
-        piv[k] = piv[j];
-        piv[j] = t;
-        S[(size_t)piv[k] * m + piv[k]] = sqrt_(v);
-      }
-    }
-    __syncthreads();
-    if (s_stop) {
-      rank = k;
-      break;
-    }
-    const int pk = piv[k];
-    const F lkk = S[(size_t)pk * m + pk];
-    for (int r = k + 1 + tid; r < m; r += nt) S[(size_t)piv[r] * m + pk] /= lkk;
-    __syncthreads();
-    const int rem = m - k - 1;
-    for (int e = tid; e < rem * rem; e += nt) {
-      const int pr = piv[k + 1 + e / rem], pc = piv[k + 1 + e % rem];
-      S[(size_t)pr * m + pc] = fma(-S[(size_t)pr * m + pk], S[(size_t)pc * m + pk], S[(size_t)pr * m + pc]);
-    }
+  for (int r = tid; r < m; r += nt) {
+    piv[r] = r;
+    d[r] = S[(size_t)r * m + r];
   }
   __syncthreads();
-  return rank;
+  F dref = F(0);
+  for (int k = 0; k < m; ++k) {
+    F v = F(-1);
+    int j = m;
+    for (int p = k + tid; p < m; p += nt) {
+      const F w = d[piv[p]];
+      if (w > v) { v = w; j = p; }
+    }
+    cta_argmax(v, j, red_v, red_i);
+    if (k == 0) dref = v;
+    if (j >= m || !(v > rank_tol * dref)) return k;
+    const int pk = piv[j], pj = piv[k];
+    const F lkk = sqrt_(v);
+    F* const col = S + (size_t)pk * m;
+    for (int p = k + 1 + tid; p < m; p += nt) {
+      const int r = p == j ? pj : piv[p];
+      F acc = col[r];
+      int c = 0;
+      for (; c + 4 <= k; c += 4) {
+        F a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const F* const q = S + (size_t)piv[c + u] * m;
+          a[u] = q[r];
+          b[u] = q[pk];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = fma(-a[u], b[u], acc);
+      }
+      for (; c < k; ++c) {
+        const F* const q = S + (size_t)piv[c] * m;
+        acc = fma(-q[r], q[pk], acc);
+      }
+      const F l = acc / lkk;
+      col[r] = l;
+      d[r] = fma(-l, l, d[r]);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      col[pk] = lkk;
+      piv[j] = pj;
+      piv[k] = pk;
+    }
+    __syncthreads();
+  }
+  return m;
 }
 
-// Normal matrix M = L'L (rank x rank) of the rank-deficient factor and its
-// Cholesky factor, by one CTA (nothing to do when rank = m).  Sets *s_bad if
-// M is not positive definite.
+// The factor by position: Q[c m + p] = L(p, c) for p >= c, from S as
+// cta_pivoted_cholesky leaves it.
 template <typename F>
-__device__ void cta_ls_prepare(const F* S, int m, const int* piv, int rank, F* M, int* s_bad) {
-  if (rank == m || rank == 0) return;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < rank * rank; e += nt) {
-    const int a = e / rank, b = e % rank;
-    if (b > a) continue;
-    F acc = 0;
-    for (int i = a; i < m; ++i) acc = fma(S[(size_t)piv[i] * m + piv[a]], S[(size_t)piv[i] * m + piv[b]], acc);
-    M[(size_t)a * rank + b] = acc;
-    M[(size_t)b * rank + a] = acc;
+__device__ void cta_by_position(const F* S, int m, const int* piv, int rank, F* Q) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int c = w; c < rank; c += nw) {
+    const F* const col = S + (size_t)piv[c] * m;
+    for (int p = c + lane; p < m; p += 32) Q[(size_t)c * m + p] = col[piv[p]];
   }
+  __syncthreads();
+}
+
+// In-place Cholesky of the n x n SPD matrix M (full symmetric storage) by one
+// CTA: column c of the factor replaces row c from the diagonal on.  Sets *s_bad on
+// a non-positive pivot (and goes on with 1 in its place).
+template <typename F>
+__device__ void cta_cholesky(F* M, int n, int* s_bad) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    F* const col = M + (size_t)k * n;
+    for (int r = k + tid; r < n; r += nt) {
+      F acc = col[r];
+      int c = 0;
+      for (; c + 4 <= k; c += 4) {
+        F a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          a[u] = M[(size_t)(c + u) * n + r];
+          b[u] = M[(size_t)(c + u) * n + k];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = fma(-a[u], b[u], acc);
+      }
+      for (; c < k; ++c) acc = fma(-M[(size_t)c * n + r], M[(size_t)c * n + k], acc);
+      col[r] = acc;
+    }
+    __syncthreads();
+    const F dkk = col[k];
+    if (!(dkk > F(0)) && tid == 0) *s_bad = 1;
+    const F lkk = sqrt_(dkk > F(0) ? dkk : F(1));
+    __syncthreads();
+    for (int r = k + tid; r < n; r += nt) col[r] = r == k ? lkk : col[r] / lkk;
+    __syncthreads();
+  }
+}
+
+// Normal matrix M = L'L (rank x rank) of a rank-deficient factor (by position)
+// and its Cholesky factor, by one CTA (nothing to do when rank = m).  Sets *s_bad
+// if M is not positive definite.  Tiles of 32 x 32 entries, their rows' columns
+// staged 32 at a time; the entries of L above its diagonal count as zeros.
+template <typename F>
+__device__ void cta_ls_prepare(const F* Q, int m, int rank, F* M, int* s_bad) {
+  if (rank == m || rank == 0) return;
+  __shared__ F ta[32][33], tb[32][33];
+  constexpr int NR = 32 / (kBwdThreads / 32);  // entries per thread
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, ny = kBwdThreads / 32;
+  for (int a0 = 0; a0 < rank; a0 += 32)
+    for (int b0 = 0; b0 <= a0; b0 += 32) {
+      F acc[NR];
+#pragma unroll
+      for (int u = 0; u < NR; ++u) acc[u] = F(0);
+      for (int i0 = a0; i0 < m; i0 += 32) {
+        const int i = i0 + x;
+#pragma unroll
+        for (int u = 0; u < NR; ++u) {
+          const int a = a0 + y + u * ny, b = b0 + y + u * ny;
+          ta[y + u * ny][x] = (a < rank && i < m && i >= a) ? Q[(size_t)a * m + i] : F(0);
+          tb[y + u * ny][x] = (b < rank && i < m && i >= b) ? Q[(size_t)b * m + i] : F(0);
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int i2 = 0; i2 < 32; ++i2)
+#pragma unroll
+          for (int u = 0; u < NR; ++u) acc[u] = fma(ta[y + u * ny][i2], tb[x][i2], acc[u]);
+        __syncthreads();
+      }
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        const int a = a0 + y + u * ny, b = b0 + x;
+        if (a < rank && b <= a) {
+          M[(size_t)a * rank + b] = acc[u];
+          M[(size_t)b * rank + a] = acc[u];
+        }
+      }
+    }
   cta_cholesky(M, rank, s_bad);
 }
 
-// Least-squares solution of S lambda = b within the range of the pivoted
-// factor (one thread; b is overwritten by lambda, tmp has m entries):
+// x <- L^{-1} x for the n x n lower triangle L(r, c) = Q[c ld + r], by one warp:
+// each solved entry is taken out of all later rows (the row sums' own order).
+template <typename F>
+__device__ void warp_forward(const F* Q, int ld, int n, F* x) {
+  const int lane = threadIdx.x & 31;
+  for (int k = 0; k < n; ++k) {
+    const F* const col = Q + (size_t)k * ld;
+    const F xk = x[k] / col[k];
+    __syncwarp();
+    if (lane == 0) x[k] = xk;
+    for (int r = k + 1 + lane; r < n; r += 32) x[r] = fma(-col[r], xk, x[r]);
+    __syncwarp();
+  }
+}
+
+// x <- L^{-T} x, by one warp.  A row's sum runs over the later rows in
+// increasing order, so it starts with the one that was solved last and is one
+// chain of multiply-adds; the lanes load its operands 32 at a time, ahead.
+template <typename F>
+__device__ void warp_backward(const F* Q, int ld, int n, F* x) {
+  const int lane = threadIdx.x & 31;
+  for (int r = n - 1; r >= 0; --r) {
+    const F* const col = Q + (size_t)r * ld;
+    F v = x[r];
+    F q = r + 1 + lane < n ? col[r + 1 + lane] : F(0), y = r + 1 + lane < n ? x[r + 1 + lane] : F(0);
+    for (int k0 = r + 1; k0 < n; k0 += 32) {
+      const F qc = q, yc = y;
+      const int kn = k0 + 32 + lane;
+      q = kn < n ? col[kn] : F(0);
+      y = kn < n ? x[kn] : F(0);
+      const int cnt = min(32, n - k0);
+#pragma unroll 4
+      for (int l = 0; l < cnt; ++l) v = fma(-shfl_f(qc, l), shfl_f(yc, l), v);
+    }
+    v = v / col[r];
+    __syncwarp();
+    if (lane == 0) x[r] = v;
+    __syncwarp();
+  }
+}
+
+// Least-squares solution of S lambda = b within the range of the pivoted factor
+// Q (by position), by one CTA (b is overwritten by lambda, tmp has m entries):
 // v minimizes |L v - b_p| (b_p = b in pivot order), lambda_p = [L11^{-T} v; 0].
 // For rank = m this is the plain solve L11^{-T} L11^{-1} b_p.
 template <typename F>
-__device__ void ls_apply_serial(const F* S, int m, const int* piv, int rank, const F* M, F* b, F* tmp) {
-  auto L = [&](int r, int c) -> F { return S[(size_t)piv[r] * m + piv[c]]; };
+__device__ void cta_ls_apply(const F* Q, int m, const int* piv, int rank, const F* M, F* b, F* tmp) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  __syncthreads();
   if (rank == m) {
-    for (int r = 0; r < m; ++r) {
-      F v = b[piv[r]];
-      for (int k = 0; k < r; ++k) v = fma(-L(r, k), tmp[k], v);
-      tmp[r] = v / L(r, r);
-    }
+    for (int p = tid; p < m; p += nt) tmp[p] = b[piv[p]];
   } else {
-    for (int a = 0; a < rank; ++a) {
+    for (int a = tid; a < rank; a += nt) {
       F acc = 0;
-      for (int i = a; i < m; ++i) acc = fma(L(i, a), b[piv[i]], acc);
+      for (int i = a; i < m; ++i) acc = fma(Q[(size_t)a * m + i], b[piv[i]], acc);
       tmp[a] = acc;
     }
-    if (rank > 0) chol_solve_serial(M, rank, tmp);
   }
-  for (int r = rank - 1; r >= 0; --r) {
-    F v = tmp[r];
-    for (int k = r + 1; k < rank; ++k) v = fma(-L(k, r), tmp[k], v);
-    tmp[r] = v / L(r, r);
+  __syncthreads();
+  if (tid < 32) {
+    if (rank == m) {
+      warp_forward(Q, m, m, tmp);
+    } else if (rank > 0) {
+      warp_forward(M, rank, rank, tmp);
+      warp_backward(M, rank, rank, tmp);
+    }
+    warp_backward(Q, m, rank, tmp);
   }
-  for (int r = 0; r < m; ++r) b[piv[r]] = r < rank ? tmp[r] : F(0);
+  __syncthreads();
+  for (int p = tid; p < m; p += nt) b[piv[p]] = p < rank ? tmp[p] : F(0);
+  __syncthreads();
 }
 
 template <typename F, int NX, int NU, int DP, bool DI>
-__global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
+__global__ void __launch_bounds__(kBwdThreads) k_bwd_main(Dev<F> D, BwdDev<F> B) {
   using CL = CacheLayout<NX, NU>;
   __shared__ Model<F, NX, NU> Mo;
-  __shared__ int s_bad;
+  __shared__ int s_bad, s_cnt;
   load_model<F, NX, NU>(Mo, D.model);
   const int sc = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const ScenMeta s = D.meta[sc];
   const BwdScen bs = B.bs[sc];
   const int N = s.N, T = s.T, P = s.P, m = bs.m;
-  if (tid == 0) s_bad = 0;
+  if (tid == 0) {
+    s_bad = 0;
+    s_cnt = 0;
+  }
   __syncthreads();
   F* cache = D.cache + s.xs_off * CL::E;
   const uint16_t* Wm = B.Wb + s.as_off;
@@ -397,98 +564,197 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
   int* piv = B.piv + s.ps_off;
   F* rhs = B.vec + bs.v_off;
   F* tmp = rhs + 2 * m;
+  F* diag = rhs + 3 * m;
   F* pos0 = B.pos0 + s.as_off * DP;
   F* force = B.force + s.as_off * DP;
   auto Q = [&](int i, int r) { return D.Qd[(s.agent_off + i) * NX + r]; };
   auto Qf = [&](int i, int r) { return D.Qfd[(s.agent_off + i) * NX + r]; };
   auto XR = [&](int i, int r) { return D.x_ref[(s.agent_off + i) * NX + r]; };
 
-  // 1. factorization of the global per-agent Hessian with the final working set
-  for (int i = tid; i < N; i += nt) {
-    F rbar[NU], qbar[NX];
-#pragma unroll
-    for (int c = 0; c < NU; ++c) rbar[c] = F(2) * D.Rd[(s.agent_off + i) * NU + c];
-#pragma unroll
-    for (int r = 0; r < NX; ++r) qbar[r] = F(2) * Q(i, r);
-    F Pn[NX][NX];
-#pragma unroll
-    for (int r = 0; r < NX; ++r)
-#pragma unroll
-      for (int c = 0; c < NX; ++c) {
-        Pn[r][c] = (r == c) ? F(2) * Qf(i, r) : F(0);
-        cache[((size_t)T * CL::E + CL::P + r * NX + c) * N + i] = Pn[r][c];
+  // Solves the LQ problem of every agent with linear term lin(i, t, r) and initial
+  // state x0(i, r), and hands out states (outx(i, t, r, x)) and inputs
+  // (outu(i, t, c, u)): one thread per axis of an agent for the double integrator,
+  // else one per agent.
+  auto solve_agents = [&](auto lin, auto x0, bool at_bounds, auto outx, auto outu) {
+    if constexpr (DI) {
+      for (int e = tid; e < N * DP; e += nt) {
+        const int c = e / N, i = e - c * N;
+        F* kk = B.kks + ((s.agent_off + i) * DP + c) * (size_t)B.kk_stride;
+        lq_axis<F, NX, NU>(Mo, cache, Wm, N, i, T, c, T, [&](int t, int r, auto pos) { return lin(i, t, r, pos); }, x0(i, c),
+                           x0(i, DP + c), at_bounds, [&](int t) -> F& { return kk[t]; },
+                           [&](int t, F xp, F xv) {
+                             outx(i, t, c, xp);
+                             outx(i, t, DP + c, xv);
+                           },
+                           [&](int t, F u) { outu(i, t, c, u); });
       }
-    int bad = 0;
-    for (int t = T - 1; t >= 0; --t) {
-      const uint16_t mask = Wm[(size_t)t * N + i];
-      F Pt[NX][NX], K[NU][NX], L[NU][NU];
-      auto put = [&](int r, int c, F v) {
-        Pt[r][c] = v;
-        Pt[c][r] = v;
-      };
-      auto putB = [](int, int, F) {};
-      bad |= factor_stage<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), Pn, mask, rbar, t >= 1 ? qbar : nullptr, 1, put, putB, K, L);
+    } else {
+      for (int i = tid; i < N; i += nt) {
+        F xs[NX];
 #pragma unroll
-      for (int r = 0; r < NU; ++r) {
+        for (int r = 0; r < NX; ++r) xs[r] = x0(i, r);
+        F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
+        lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T,
+                                [&](int t, int r) { return lin(i, t, r, r < DP); }, xs, at_bounds, kk,
+                                [&](int t, const F (&x)[NX]) {
 #pragma unroll
-        for (int c = 0; c < NX; ++c) cache[((size_t)t * CL::E + CL::K + r * NX + c) * N + i] = K[r][c];
+                                  for (int r = 0; r < NX; ++r) outx(i, t, r, x[r]);
+                                },
+                                [&](int t, const F (&u)[NU]) {
 #pragma unroll
-        for (int c = 0; c <= r; ++c) cache[((size_t)t * CL::E + CL::L + r * NU + c) * N + i] = L[r][c];
-      }
-      if (t >= 1) {
-#pragma unroll
-        for (int r = 0; r < NX; ++r)
-#pragma unroll
-          for (int c = 0; c < NX; ++c) {
-            cache[((size_t)t * CL::E + CL::P + r * NX + c) * N + i] = Pt[r][c];
-            Pn[r][c] = Pt[r][c];
-          }
+                                  for (int c = 0; c < NU; ++c) outu(i, t, c, u[c]);
+                                });
       }
     }
-    if (bad) atomicOr(&s_bad, 1);
+    __syncthreads();
+  };
+  auto no_input = [](int, int, int, F) {};
+  auto zero0 = [](int, int) { return F(0); };
+  auto init0 = [&](int i, int r) { return D.x_init[(s.agent_off + i) * NX + r]; };
+  // positions of every step t >= 1, the base of a right-hand side
+  auto to_pos0 = [&](int i, int t, int r, F x) {
+    if (t >= 1 && r < DP) pos0[((size_t)i * T + (t - 1)) * DP + r] = x;
+  };
+
+  // 1. factorization of the global per-agent Hessian with the final working set
+  if constexpr (DI) {
+    // one lane per axis, as many agents of a warp as fit
+    using AC = AgentConst<NX, NU>;
+    constexpr int NG = 32 / DP, kRun = NG * (kBwdThreads / 32);
+    __shared__ F kct[AC::KC * kRun];
+    const int lane = tid & 31, g = lane / DP;
+    for (int i0 = 0; i0 < N; i0 += kRun) {
+      const int q = (tid >> 5) * NG + g, i = i0 + q;
+      const bool mine = g < NG && i < N;
+      AxisView<F, NX, NU, DP, 1> V;
+      V.N = N;
+      V.T = T;
+      V.ks = kRun;
+      V.nc = 0;
+      V.c0 = mine ? lane - g * DP : 0;
+      V.rho = F(0);
+      const int64_t ag = s.agent_off + (mine ? i : 0);
+      V.cache = cache + V.c0 * N + (mine ? i : 0);
+      V.Wm = B.Wb + s.as_off + (mine ? i : 0);
+      V.Cm = D.Cm + s.as_off + (mine ? i : 0);
+      V.Us = nullptr;
+      V.Xo = nullptr;
+      V.h = nullptr;
+      V.xr = nullptr;
+      V.xi = nullptr;
+      V.qf = D.Qfd + ag * NX + V.c0;
+      V.kc = kct + (mine ? q : 0) + V.c0 * kRun;
+      axis_model(V, Mo);
+      if (mine) {
+        kct[(AC::RB + V.c0) * kRun + q] = F(2) * D.Rd[ag * NU + V.c0];
+        kct[(AC::QB + V.c0) * kRun + q] = F(2) * Q(i, V.c0);
+        kct[(AC::QB + DP + V.c0) * kRun + q] = F(2) * Q(i, DP + V.c0);
+      }
+      __syncwarp();
+      if (axis_factor<false>(V, mine, T - 1, mine ? g * DP : 0)) atomicOr(&s_bad, 1);
+      __syncwarp();
+    }
+    __syncthreads();
     // the forward factor cache no longer matches: force a refactorization on the next solve
-    for (int t = 0; t < T; ++t) D.Cm[s.as_off + (size_t)t * N + i] = 0xFFFF;
+    for (int e = tid; e < N * T; e += nt) D.Cm[s.as_off + e] = 0xFFFF;
+  } else {
+    for (int i = tid; i < N; i += nt) {
+      F rbar[NU], qbar[NX];
+#pragma unroll
+      for (int c = 0; c < NU; ++c) rbar[c] = F(2) * D.Rd[(s.agent_off + i) * NU + c];
+#pragma unroll
+      for (int r = 0; r < NX; ++r) qbar[r] = F(2) * Q(i, r);
+      F Pn[NX][NX];
+#pragma unroll
+      for (int r = 0; r < NX; ++r)
+#pragma unroll
+        for (int c = 0; c < NX; ++c) {
+          Pn[r][c] = (r == c) ? F(2) * Qf(i, r) : F(0);
+          cache[((size_t)T * CL::E + CL::P + r * NX + c) * N + i] = Pn[r][c];
+        }
+      int bad = 0;
+      for (int t = T - 1; t >= 0; --t) {
+        const uint16_t mask = Wm[(size_t)t * N + i];
+        F Pt[NX][NX], K[NU][NX], L[NU][NU];
+        auto put = [&](int r, int c, F v) {
+          Pt[r][c] = v;
+          Pt[c][r] = v;
+        };
+        auto putB = [](int, int, F) {};
+        bad |= factor_stage<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), Pn, mask, rbar, t >= 1 ? qbar : nullptr, 1, put, putB, K, L);
+#pragma unroll
+        for (int r = 0; r < NU; ++r) {
+#pragma unroll
+          for (int c = 0; c < NX; ++c) cache[((size_t)t * CL::E + CL::K + r * NX + c) * N + i] = K[r][c];
+#pragma unroll
+          for (int c = 0; c <= r; ++c) cache[((size_t)t * CL::E + CL::L + r * NU + c) * N + i] = L[r][c];
+        }
+        if (t >= 1) {
+#pragma unroll
+          for (int r = 0; r < NX; ++r)
+#pragma unroll
+            for (int c = 0; c < NX; ++c) {
+              cache[((size_t)t * CL::E + CL::P + r * NX + c) * N + i] = Pt[r][c];
+              Pn[r][c] = Pt[r][c];
+            }
+        }
+      }
+      if (bad) atomicOr(&s_bad, 1);
+      // the forward factor cache no longer matches: force a refactorization on the next solve
+      for (int t = 0; t < T; ++t) D.Cm[s.as_off + (size_t)t * N + i] = 0xFFFF;
+    }
   }
   __syncthreads();
 
-  const F zero0[NX] = {};
   // 2. position responses to unit forces at the agent's active times
-  for (int task = tid; task < N * DP; task += nt) {
-    const int i = task / DP, cin = task % DP;
-    const unsigned long long msk = B.amask[s.agent_off + i];
-    F* kk = B.kks + ((s.agent_off + i) * DP + cin) * (size_t)B.kk_stride;
-    for (int tp = 1; tp <= T; ++tp) {
-      if (!((msk >> (tp - 1)) & 1ull)) continue;
-      auto lin = [&](int t, int r) -> F { return (t == tp && r == cin) ? F(-1) : F(0); };
-      auto outx = [&](int t, const F (&x)[NX]) {
-        if (t >= 1) {
+  if constexpr (DI) {
+    // (agent, step) of every response, listed in the force block (written later)
+    int* const list = reinterpret_cast<int*>(force);
+    for (int i = tid; i < N; i += nt) {
+      unsigned long long msk = B.amask[s.agent_off + i];
+      int at = msk ? atomicAdd(&s_cnt, __popcll(msk)) : 0;
+      for (; msk; msk &= msk - 1) list[at++] = i | (__ffsll((long long)msk) - 1) << 16;
+    }
+    __syncthreads();
+    const int nr = s_cnt;
+    for (int e = tid; e < nr * DP; e += nt) {
+      const int c = e / nr, i = list[e - c * nr] & 0xFFFF, tp = (list[e - c * nr] >> 16) + 1;
+      // a response moves its own axis only; a word of another axis holds the gains
+      F* const out = psi + (((size_t)i * T + (tp - 1)) * DP + c) * T * DP;
+      const int other = c == 0 ? 1 : 0;
+      lq_axis<F, NX, NU>(Mo, cache, Wm, N, i, T, c, tp,
+                         [&](int t, int, auto pos) { return (pos && t == tp) ? F(-1) : F(0); }, F(0), F(0), false,
+                         [&](int t) -> F& { return out[t * DP + other]; },
+                         [&](int t, F xp, F) {
+                           if (t >= 1) out[(t - 1) * DP + c] = xp;
+                         },
+                         [](int, F) {});
+    }
+  } else {
+    const F z0[NX] = {};
+    for (int task = tid; task < N * DP; task += nt) {
+      const int i = task / DP, cin = task % DP;
+      const unsigned long long msk = B.amask[s.agent_off + i];
+      F* kk = B.kks + ((s.agent_off + i) * DP + cin) * (size_t)B.kk_stride;
+      for (int tp = 1; tp <= T; ++tp) {
+        if (!((msk >> (tp - 1)) & 1ull)) continue;
+        auto lin = [&](int t, int r) -> F { return (t == tp && r == cin) ? F(-1) : F(0); };
+        auto outx = [&](int t, const F (&x)[NX]) {
+          if (t >= 1) {
 #pragma unroll
-          for (int c = 0; c < DP; ++c)
-            psi[((((size_t)i * T + (tp - 1)) * DP + cin) * T + (t - 1)) * DP + c] = x[c];
-        }
-      };
-      auto outu = [&](int, const F (&)[NU]) {};
-      lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, zero0, false, kk, outx, outu);
+            for (int c = 0; c < DP; ++c)
+              psi[((((size_t)i * T + (tp - 1)) * DP + cin) * T + (t - 1)) * DP + c] = x[c];
+          }
+        };
+        auto outu = [&](int, const F (&)[NU]) {};
+        lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, z0, false, kk, outx, outu);
+      }
     }
   }
   __syncthreads();
   // 3. base solution (cost terms only) for the right-hand side of S mu = d - G z0
-  for (int i = tid; i < N; i += nt) {
-    F x0[NX];
-#pragma unroll
-    for (int r = 0; r < NX; ++r) x0[r] = D.x_init[(s.agent_off + i) * NX + r];
-    F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
-    auto lin = [&](int t, int r) -> F { return (F(-2) * (t < T ? Q(i, r) : Qf(i, r))) * XR(i, r); };
-    auto outx = [&](int t, const F (&x)[NX]) {
-      if (t >= 1) {
-#pragma unroll
-        for (int c = 0; c < DP; ++c) pos0[((size_t)i * T + (t - 1)) * DP + c] = x[c];
-      }
-    };
-    auto outu = [&](int, const F (&)[NU]) {};
-    lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, x0, true, kk, outx, outu);
-  }
-  __syncthreads();
+  auto cost = [&](int i, int t, int r, auto) -> F { return (F(-2) * (t < T ? Q(i, r) : Qf(i, r))) * XR(i, r); };
+  solve_agents(cost, init0, true, to_pos0, no_input);
 
   // 4. Schur complement S_hk = sum over shared agents of sigma sigma a_h' Psi a_k
   auto hs = [&](int h, int& i, int& j, int& tm1, int& pair) {
@@ -520,6 +786,7 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
         const F ak = a[((size_t)tk * DP + cin) * P + pk2];
 #pragma unroll
         for (int cout = 0; cout < DP; ++cout) {
+          if (DI && cout != cin) continue;  // the axes do not respond to one another
           const F ah = a[((size_t)th * DP + cout) * P + ph];
           v = fma(ah * psi[((((size_t)ma * T + tk) * DP + cin) * T + th) * DP + cout], ak, v);
         }
@@ -541,18 +808,28 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
   }
   // 5. rank-revealing factorization of S; least-squares multipliers mu
   __syncthreads();
-  const int rank = m > 0 ? cta_pivoted_cholesky(Sm, m, piv, F(B.rank_tol)) : 0;
-  if (m > 0) cta_ls_prepare(Sm, m, piv, rank, Mn, &s_bad);
+  const int rank = m > 0 ? cta_pivoted_cholesky(Sm, m, piv, diag, F(B.rank_tol)) : 0;
   __syncthreads();
-  if (tid == 0 && m > 0) ls_apply_serial(Sm, m, piv, rank, Mn, rhs, tmp);
-  __syncthreads();
+  if (m > 0) {
+    // the factor by position in the second block; the normal matrix in the first
+    cta_by_position(Sm, m, piv, rank, Mn);
+    cta_ls_prepare(Mn, m, rank, Sm, &s_bad);
+    cta_ls_apply(Mn, m, piv, rank, Sm, rhs, tmp);
+  }
 
   // 6. coupling forces G' mu, polished primal solve
   auto forces = [&](const F* lam) {
     for (int e = tid; e < N * T * DP; e += nt) force[e] = 0;
     __syncthreads();
-    if (tid == 0) {
-      for (int h = 0; h < m; ++h) {
+    // the active rows are sorted by step: one thread per step, in their order
+    for (int t = tid; t < T; t += nt) {
+      int lo = 0, hi = m;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (act[mid] < t * P) lo = mid + 1;
+        else hi = mid;
+      }
+      for (int h = lo; h < m && act[h] < (t + 1) * P; ++h) {
         int i, j, tm1, pair;
         hs(h, i, j, tm1, pair);
 #pragma unroll
@@ -566,29 +843,14 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
     __syncthreads();
   };
   forces(rhs);
-  for (int i = tid; i < N; i += nt) {
-    F x0[NX];
-#pragma unroll
-    for (int r = 0; r < NX; ++r) x0[r] = D.x_init[(s.agent_off + i) * NX + r];
-    F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
-    auto lin = [&](int t, int r) -> F {
-      F v = (F(-2) * (t < T ? Q(i, r) : Qf(i, r))) * XR(i, r);
-      if (r < DP) v -= force[((size_t)i * T + (t - 1)) * DP + r];
-      return v;
-    };
-    F* Xp = B.Xp + (s.xs_off + (int64_t)i * (T + 1)) * NX;
-    F* Up = B.Up + (s.as_off + (int64_t)i * T) * NU;
-    auto outx = [&](int t, const F (&x)[NX]) {
-#pragma unroll
-      for (int r = 0; r < NX; ++r) Xp[(size_t)t * NX + r] = x[r];
-    };
-    auto outu = [&](int t, const F (&u)[NU]) {
-#pragma unroll
-      for (int c = 0; c < NU; ++c) Up[(size_t)t * NU + c] = u[c];
-    };
-    lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, x0, true, kk, outx, outu);
-  }
-  __syncthreads();
+  solve_agents(
+      [&](int i, int t, int r, auto pos) -> F {
+        F v = cost(i, t, r, pos);
+        if (pos) v -= force[((size_t)i * T + (t - 1)) * DP + r];
+        return v;
+      },
+      init0, true, [&](int i, int t, int r, F x) { B.Xp[(s.xs_off + (int64_t)i * (T + 1) + t) * NX + r] = x; },
+      [&](int i, int t, int c, F u) { B.Up[(s.as_off + (int64_t)i * T + t) * NU + c] = u; });
 
   F* lamw = rhs + m;
   if (!B.adjoint) {
@@ -601,20 +863,8 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
     return;
   }
   // 7. adjoint: w0 = H^{-1} dl/dz (homogeneous), S lam = -G w0, w = w0 + Psi G' lam
-  for (int i = tid; i < N; i += nt) {
-    const double* g = B.gX + (s.xs_off + (int64_t)i * (T + 1)) * NX;
-    F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
-    auto lin = [&](int t, int r) -> F { return -F(g[(size_t)t * NX + r]); };
-    auto outx = [&](int t, const F (&x)[NX]) {
-      if (t >= 1) {
-#pragma unroll
-        for (int c = 0; c < DP; ++c) pos0[((size_t)i * T + (t - 1)) * DP + c] = x[c];
-      }
-    };
-    auto outu = [&](int, const F (&)[NU]) {};
-    lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, zero0, false, kk, outx, outu);
-  }
-  __syncthreads();
+  auto loss = [&](int i, int t, int r, auto) -> F { return -F(B.gX[(s.xs_off + (int64_t)i * (T + 1) + t) * NX + r]); };
+  solve_agents(loss, zero0, false, to_pos0, no_input);
   for (int h = tid; h < m; h += nt) {
     int i, j, tm1, pair;
     hs(h, i, j, tm1, pair);
@@ -626,30 +876,16 @@ __global__ void __launch_bounds__(128) k_bwd_main(Dev<F> D, BwdDev<F> B) {
     lamw[h] = v;
   }
   __syncthreads();
-  if (tid == 0 && m > 0) ls_apply_serial(Sm, m, piv, rank, Mn, lamw, tmp);
-  __syncthreads();
+  if (m > 0) cta_ls_apply(Mn, m, piv, rank, Sm, lamw, tmp);
   forces(lamw);
-  for (int i = tid; i < N; i += nt) {
-    const double* g = B.gX + (s.xs_off + (int64_t)i * (T + 1)) * NX;
-    F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
-    auto lin = [&](int t, int r) -> F {
-      F v = -F(g[(size_t)t * NX + r]);
-      if (r < DP) v -= force[((size_t)i * T + (t - 1)) * DP + r];
-      return v;
-    };
-    F* Wx = B.Wx + (s.xs_off + (int64_t)i * (T + 1)) * NX;
-    F* Wu = B.Wu + (s.as_off + (int64_t)i * T) * NU;
-    auto outx = [&](int t, const F (&x)[NX]) {
-#pragma unroll
-      for (int r = 0; r < NX; ++r) Wx[(size_t)t * NX + r] = x[r];
-    };
-    auto outu = [&](int t, const F (&u)[NU]) {
-#pragma unroll
-      for (int c = 0; c < NU; ++c) Wu[(size_t)t * NU + c] = u[c];
-    };
-    lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, zero0, false, kk, outx, outu);
-  }
-  __syncthreads();
+  solve_agents(
+      [&](int i, int t, int r, auto pos) -> F {
+        F v = loss(i, t, r, pos);
+        if (pos) v -= force[((size_t)i * T + (t - 1)) * DP + r];
+        return v;
+      },
+      zero0, false, [&](int i, int t, int r, F x) { B.Wx[(s.xs_off + (int64_t)i * (T + 1) + t) * NX + r] = x; },
+      [&](int i, int t, int c, F u) { B.Wu[(s.as_off + (int64_t)i * T + t) * NU + c] = u; });
 
   // 8. gradients: dl/dtheta = -w' (dH/dtheta z + dg/dtheta)
   for (int i = tid; i < N; i += nt) {
@@ -731,67 +967,110 @@ __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
     s_idx = LLONG_MAX;
   }
   __syncthreads();
-  // Costates of agent i backwards from lambda_{T+1} = 0; for every input u_{t-1}
-  // visit(t-1, c, working-set mask, u, g) with g = 2 R u_{t-1} + B' lambda_t.
-  auto sweep = [&](int i, auto&& visit) {
-    const Model<F, NX, NU>& Ma = agent_model<F, NX, NU>(D, Mo, s, i);
-    const F* Xp = B.Xp + (s.xs_off + (int64_t)i * (T + 1)) * NX;
-    const F* Up = B.Up + (s.as_off + (int64_t)i * T) * NU;
-    F lam[NX];
-#pragma unroll
-    for (int r = 0; r < NX; ++r) lam[r] = F(0);
-    for (int t = T; t >= 1; --t) {
-      F ln[NX];
-#pragma unroll
-      for (int r = 0; r < NX; ++r) {
-        const F q = t < T ? D.Qd[(s.agent_off + i) * NX + r] : D.Qfd[(s.agent_off + i) * NX + r];
-        F acc = (F(2) * q) * (Xp[(size_t)t * NX + r] - D.x_ref[(s.agent_off + i) * NX + r]);
-        if (r < DP) acc -= force[((size_t)i * T + (t - 1)) * DP + r];
-#pragma unroll
-        for (int k = 0; k < NX; ++k) acc = fma(Ma.A[k][r], lam[k], acc);
-        ln[r] = acc;
+  // g = 2 R u_t + B' lambda_{t+1} of every input, from the costates backwards from
+  // lambda_{T+1} = 0, kept in the adjoint's input block (unused in these rounds):
+  // one thread per axis of an agent for the double integrator, else per agent
+  F* const G = B.Wu + s.as_off * NU;
+  if constexpr (DI) {
+    constexpr int H = NU;
+    const F one = Mo.A[0][0], dt = Mo.A[0][H], b1 = Mo.B[0][0], b2 = Mo.B[H][0];
+    for (int e = tid; e < N * H; e += nt) {
+      const int c = e / N, i = e - c * N;
+      const int64_t ag = s.agent_off + i;
+      const F* Xp = B.Xp + (s.xs_off + (int64_t)i * (T + 1)) * NX;
+      const F* Up = B.Up + (s.as_off + (int64_t)i * T) * NU;
+      F lp = F(0), lv = F(0);
+      for (int t = T; t >= 1; --t) {
+        const F* const w = (t < T ? D.Qd : D.Qfd) + ag * NX;
+        F np = (F(2) * w[c]) * (Xp[(size_t)t * NX + c] - D.x_ref[ag * NX + c]);
+        np -= force[((size_t)i * T + (t - 1)) * DP + c];
+        const F nv = (F(2) * w[H + c]) * (Xp[(size_t)t * NX + H + c] - D.x_ref[ag * NX + H + c]);
+        lv = fma(one, lv, fma(dt, lp, nv));
+        lp = fma(one, lp, np);
+        const F g = (F(2) * D.Rd[ag * NU + c]) * Up[(size_t)(t - 1) * NU + c];
+        G[((size_t)i * T + (t - 1)) * NU + c] = fma(b2, lv, fma(b1, lp, g));
       }
-      const uint16_t msk = Wb[(size_t)(t - 1) * N + i];
+    }
+  } else {
+    for (int i = tid; i < N; i += nt) {
+      const Model<F, NX, NU>& Ma = agent_model<F, NX, NU>(D, Mo, s, i);
+      const F* Xp = B.Xp + (s.xs_off + (int64_t)i * (T + 1)) * NX;
+      const F* Up = B.Up + (s.as_off + (int64_t)i * T) * NU;
+      F lam[NX];
 #pragma unroll
-      for (int c = 0; c < NU; ++c) {
-        const F u = Up[(size_t)(t - 1) * NU + c];
-        F g = (F(2) * D.Rd[(s.agent_off + i) * NU + c]) * u;
+      for (int r = 0; r < NX; ++r) lam[r] = F(0);
+      for (int t = T; t >= 1; --t) {
+        F ln[NX];
 #pragma unroll
-        for (int r = 0; r < NX; ++r) g = fma(Ma.B[r][c], ln[r], g);
-        visit(t - 1, c, msk, u, g, Ma);
+        for (int r = 0; r < NX; ++r) {
+          const F q = t < T ? D.Qd[(s.agent_off + i) * NX + r] : D.Qfd[(s.agent_off + i) * NX + r];
+          F acc = (F(2) * q) * (Xp[(size_t)t * NX + r] - D.x_ref[(s.agent_off + i) * NX + r]);
+          if (r < DP) acc -= force[((size_t)i * T + (t - 1)) * DP + r];
+#pragma unroll
+          for (int k = 0; k < NX; ++k) acc = fma(Ma.A[k][r], lam[k], acc);
+          ln[r] = acc;
+        }
+#pragma unroll
+        for (int c = 0; c < NU; ++c) {
+          F g = (F(2) * D.Rd[(s.agent_off + i) * NU + c]) * Up[(size_t)(t - 1) * NU + c];
+#pragma unroll
+          for (int r = 0; r < NX; ++r) g = fma(Ma.B[r][c], ln[r], g);
+          G[((size_t)i * T + (t - 1)) * NU + c] = g;
+        }
+#pragma unroll
+        for (int r = 0; r < NX; ++r) lam[r] = ln[r];
       }
-#pragma unroll
-      for (int r = 0; r < NX; ++r) lam[r] = ln[r];
+    }
+  }
+  __syncthreads();
+  // visit(index, i, t, c, working-set mask) for every input, agents, then steps, then components
+  const int nin = N * T * NU;
+  auto inputs = [&](auto&& visit) {
+    for (int e = tid; e < nin; e += nt) {
+      const int c = e % NU, it = e / NU, t = it % T, i = it / T;
+      visit(e, i, t, c, Wb[(size_t)t * N + i]);
     }
   };
   auto bound_mu = [](uint16_t msk, int c, F g) -> F { return (msk & (1u << c)) ? g : -g; };
   auto held = [](uint16_t msk, int c) -> bool { return (msk & (0x101u << c)) != 0; };
   // largest |multiplier|
-  for (int i = tid; i < N; i += nt)
-    sweep(i, [&](int, int c, uint16_t msk, F, F g, const Model<F, NX, NU>&) {
-      if (held(msk, c)) atomicMax(&s_scale, abs_bits(bound_mu(msk, c, g)));
+  {
+    unsigned long long top = 0;
+    inputs([&](int e, int, int, int c, uint16_t msk) {
+      if (held(msk, c)) {
+        const unsigned long long v = abs_bits(bound_mu(msk, c, G[e]));
+        top = v > top ? v : top;
+      }
     });
-  for (int h = tid; h < m; h += nt) atomicMax(&s_scale, abs_bits(mu[h]));
+    for (int h = tid; h < m; h += nt) {
+      const unsigned long long v = abs_bits(mu[h]);
+      top = v > top ? v : top;
+    }
+    if (top) atomicMax(&s_scale, top);
+  }
   __syncthreads();
   const F tol = F(B.kkt_tol);
   const F mtol = tol * from_bits(s_scale, F(0));
   // 1. the most negative multiplier (smallest order key), then its lowest index
-  for (int h = tid; h < m; h += nt)
-    if (mu[h] < -mtol) atomicMin(&s_key, mono_key(mu[h]));
-  for (int i = tid; i < N; i += nt)
-    sweep(i, [&](int, int c, uint16_t msk, F, F g, const Model<F, NX, NU>&) {
-      if (held(msk, c) && bound_mu(msk, c, g) < -mtol) atomicMin(&s_key, mono_key(bound_mu(msk, c, g)));
+  {
+    unsigned long long low = ~0ull;
+    for (int h = tid; h < m; h += nt)
+      if (mu[h] < -mtol) low = min(low, mono_key(mu[h]));
+    inputs([&](int e, int, int, int c, uint16_t msk) {
+      if (held(msk, c) && bound_mu(msk, c, G[e]) < -mtol) low = min(low, mono_key(bound_mu(msk, c, G[e])));
     });
+    if (low != ~0ull) atomicMin(&s_key, low);
+  }
   __syncthreads();
   const unsigned long long kdrop = s_key;
   if (kdrop != ~0ull) {
+    long long at = LLONG_MAX;
     for (int h = tid; h < m; h += nt)
-      if (mono_key(mu[h]) == kdrop) atomicMin(&s_idx, (long long)h);
-    for (int i = tid; i < N; i += nt)
-      sweep(i, [&](int t, int c, uint16_t msk, F, F g, const Model<F, NX, NU>&) {
-        if (held(msk, c) && mono_key(bound_mu(msk, c, g)) == kdrop)
-          atomicMin(&s_idx, (long long)m + ((long long)i * T + t) * NU + c);
-      });
+      if (mono_key(mu[h]) == kdrop) at = min(at, (long long)h);
+    inputs([&](int e, int, int, int c, uint16_t msk) {
+      if (held(msk, c) && mono_key(bound_mu(msk, c, G[e])) == kdrop) at = min(at, (long long)m + e);
+    });
+    if (at != LLONG_MAX) atomicMin(&s_idx, at);
     __syncthreads();
     if (tid == 0) {
       const long long e = s_idx;
@@ -823,31 +1102,41 @@ __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
     const F vl = (lo - u) / sl, vh = (u - hi) / sh;
     return vl > vh ? vl : vh;
   };
-  for (int64_t q = tid; q < PT; q += nt)
-    if (!hm[q]) {
-      const F v = -slack_rel(q);
-      if (v > tol) atomicMin(&s_key, ~mono_key(v));
-    }
-  for (int i = tid; i < N; i += nt)
-    sweep(i, [&](int, int c, uint16_t msk, F u, F, const Model<F, NX, NU>& Ma) {
+  const F* const Up = B.Up + s.as_off * NU;
+  auto box_of = [&](int e, int i, int c) -> F {
+    const Model<F, NX, NU>& Ma = DI ? Mo : agent_model<F, NX, NU>(D, Mo, s, i);
+    return box_rel(Up[e], Ma.umin[c], Ma.umax[c]);
+  };
+  {
+    unsigned long long low = ~0ull;
+    for (int64_t q = tid; q < PT; q += nt)
+      if (!hm[q]) {
+        const F v = -slack_rel(q);
+        if (v > tol) low = min(low, ~mono_key(v));
+      }
+    inputs([&](int e, int i, int, int c, uint16_t msk) {
       if (!held(msk, c)) {
-        const F v = box_rel(u, Ma.umin[c], Ma.umax[c]);
-        if (v > tol) atomicMin(&s_key, ~mono_key(v));
+        const F v = box_of(e, i, c);
+        if (v > tol) low = min(low, ~mono_key(v));
       }
     });
+    if (low != ~0ull) atomicMin(&s_key, low);
+  }
   __syncthreads();
   const unsigned long long kadd = s_key;
   if (kadd == ~0ull) {
     if (tid == 0) B.pchg[sc] = 0;   // KKT conditions hold
     return;
   }
-  for (int64_t q = tid; q < PT; q += nt)
-    if (!hm[q] && ~mono_key(-slack_rel(q)) == kadd) atomicMin(&s_idx, (long long)q);
-  for (int i = tid; i < N; i += nt)
-    sweep(i, [&](int t, int c, uint16_t msk, F u, F, const Model<F, NX, NU>& Ma) {
-      if (!held(msk, c) && ~mono_key(box_rel(u, Ma.umin[c], Ma.umax[c])) == kadd)
-        atomicMin(&s_idx, PT + ((long long)i * T + t) * NU + c);
+  {
+    long long at = LLONG_MAX;
+    for (int64_t q = tid; q < PT; q += nt)
+      if (!hm[q] && ~mono_key(-slack_rel(q)) == kadd) at = min(at, (long long)q);
+    inputs([&](int e, int i, int, int c, uint16_t msk) {
+      if (!held(msk, c) && ~mono_key(box_of(e, i, c)) == kadd) at = min(at, (long long)PT + e);
     });
+    if (at != LLONG_MAX) atomicMin(&s_idx, at);
+  }
   __syncthreads();
   if (tid == 0) {
     const long long e = s_idx;

@@ -1133,7 +1133,7 @@ static int bwd_solve(tadmm_handle* h, BwdDev<F>& B, std::vector<BwdScen>& bs, cu
   Dev<F> D = make_dev<F>(h);
   BwdBufs& b = h->bwd;
   int rc;
-  k_bwd_count<F, NX, NU, DP><<<h->n_scen, 32, 0, st>>>(D, B);
+  k_bwd_count<F, NX, NU, DP><<<h->n_scen, kBwdThreads, 0, st>>>(D, B);
   if ((rc = cuda_check(cudaGetLastError(), "backward count launch"))) return rc;
   std::vector<int32_t> cnt(h->n_scen);
   if ((rc = cuda_check(cudaMemcpyAsync(cnt.data(), b.cnt, 4 * h->n_scen, cudaMemcpyDeviceToHost, st), "counts")) ||
@@ -1145,7 +1145,7 @@ static int bwd_solve(tadmm_handle* h, BwdDev<F>& B, std::vector<BwdScen>& bs, cu
     bs[s].s_off = s_total;
     bs[s].v_off = v_total;
     s_total += 2 * (int64_t)cnt[s] * cnt[s];   // S, then the normal matrix of a rank-deficient S
-    v_total += 3 * (int64_t)cnt[s];
+    v_total += 4 * (int64_t)cnt[s];
   }
   auto grow = [&](void** p, size_t& cap, size_t bytes) -> int {
     if (bytes <= cap && *p) return TADMM_OK;
@@ -1169,9 +1169,9 @@ static int bwd_solve(tadmm_handle* h, BwdDev<F>& B, std::vector<BwdScen>& bs, cu
                        "backward sizes")))
     return rc;
   if (h->di)
-    k_bwd_main<F, NX, NU, DP, true><<<h->n_scen, 128, 0, st>>>(D, B);
+    k_bwd_main<F, NX, NU, DP, true><<<h->n_scen, kBwdThreads, 0, st>>>(D, B);
   else
-    k_bwd_main<F, NX, NU, DP, false><<<h->n_scen, 128, 0, st>>>(D, B);
+    k_bwd_main<F, NX, NU, DP, false><<<h->n_scen, kBwdThreads, 0, st>>>(D, B);
   return cuda_check(cudaGetLastError(), "backward launch");
 }
 
