@@ -1879,6 +1879,7 @@ struct GroupStage {
   uint8_t mem[kGroupPairs];     // member of every flattened pair
   F pos[DP][kGroupMax];         // positions p^{k+1} of the group's agents at the current step
   F sxs[DP][kGroupMax];         // over-relaxation: agent parts s^k of the consensus copies at that step
+  uint8_t amem[kGroupMax];      // member of every agent
   float posf[DP][kGroupMax];    // float64: the positions for the float32 test
   uint32_t on[kGroupMax];       // places of the agent's partners with a coupling weight at the current step
   uint16_t list[kGroupPairs];   // float64: pairs of the current step that need the projection
@@ -1961,7 +1962,7 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
   const F al = F(D.alpha), om = F(1.0 - D.alpha);
   const bool mine = my_m >= 0 && gs.active[my_m];
   const F* Xm = nullptr;
-  F* Sm = nullptr;
+  const F* Sm = nullptr;
   int Nm = 1;
   if (mine) {
     const ScenMeta& s = gs.meta[my_m];
@@ -2023,29 +2024,25 @@ __device__ void group_relaxed_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, 
       if (sv > gs.sb[m]) atomicMax(&gs.sb[m], sv);
     }
     __syncthreads();
-    if (mine) {
-      const ScenMeta& s = gs.meta[my_m];
-      const int N = s.N, i = my_i, base = gs.poff[my_m];
-      const F nc = F(agent_nc(D, s, i));
-      F sn[DP], acc[DP];
-#pragma unroll
-      for (int c = 0; c < DP; ++c) {
-        sn[c] = fma(al, st.pos[c][my_a], om * st.sxs[c][my_a]);
-        acc[c] = nc * sn[c];
-      }
+    // Every agent sums over all its partners here, so this is as long as the
+    // projection of a CTA of four warps if one lane takes all of an agent's
+    // components: one thread each (512 scenarios, 150 iterations: 169 -> 162 ms).
+    for (int e0 = tid; e0 < gs.nA * DP; e0 += nt) {
+      const int c = e0 / gs.nA, ag = e0 - c * gs.nA, m = st.amem[ag];
+      if (!gs.active[m]) continue;
+      const ScenMeta& s = gs.meta[m];
+      const int N = s.N, i = ag - gs.aoff[m], base = gs.poff[m];
+      const F sn = fma(al, st.pos[c][ag], om * st.sxs[c][ag]);
+      F acc = F(agent_nc(D, s, i)) * sn;
       for_partners(D, s, i, [&](int lp, bool first) {
         const int pair = base + lp;
         F e = smE[pair];
         if (!first) e = -e;
-#pragma unroll
-        for (int c = 0; c < DP; ++c) acc[c] = fma(e, smA[c * nP + pair], acc[c]);
+        acc = fma(e, smA[c * nP + pair], acc);
       });
-      F* h = D.h + s.as_off * DP;
-#pragma unroll
-      for (int c = 0; c < DP; ++c) {
-        h[((size_t)tm1 * DP + c) * N + i] = acc[c];
-        Sm[((size_t)tm1 * DP + c) * N + i] = sn[c];
-      }
+      const size_t q = s.as_off * DP + ((size_t)tm1 * DP + c) * N + i;
+      D.h[q] = acc;
+      D.sx[q] = sn;
     }
     __syncthreads();
   }
@@ -2274,6 +2271,7 @@ __device__ void run_group(const Dev<F>& D, const Model<F, NX, NU>& M, const int*
   const int my_a = slot < nA ? slot : -1;  // in the group
   const int my_m = my_a >= 0 ? member_of(gs.aoff, G, my_a) : -1;
   const int my_i = my_a >= 0 ? my_a - gs.aoff[my_m] : 0;
+  if (my_a >= 0) st.amem[my_a] = (uint8_t)my_m;
   bool stale = true;  // none of the agent's cached factors matches
   unsigned long long neqp = 0, nfact = 0;
   F* smE = sm;
