@@ -946,7 +946,9 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_main(Dev<F> D, BwdDev<F> B)
 template <typename F, int NX, int NU, int DP, bool DI>
 __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
   __shared__ Model<F, NX, NU> Mo;
-  __shared__ unsigned long long s_scale, s_key;
+  // one key per search: a late warp may still read the first search's when the
+  // second search writes
+  __shared__ unsigned long long s_scale, s_drop, s_add;
   __shared__ long long s_idx;
   load_model<F, NX, NU>(Mo, D.model);
   const int sc = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
@@ -963,7 +965,7 @@ __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
   const int64_t PT = (int64_t)P * T;
   if (tid == 0) {
     s_scale = ord_bits(F(1));
-    s_key = ~0ull;
+    s_drop = s_add = ~0ull;
     s_idx = LLONG_MAX;
   }
   __syncthreads();
@@ -1059,10 +1061,10 @@ __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
     inputs([&](int e, int, int, int c, uint16_t msk) {
       if (held(msk, c) && bound_mu(msk, c, G[e]) < -mtol) low = min(low, mono_key(bound_mu(msk, c, G[e])));
     });
-    if (low != ~0ull) atomicMin(&s_key, low);
+    if (low != ~0ull) atomicMin(&s_drop, low);
   }
   __syncthreads();
-  const unsigned long long kdrop = s_key;
+  const unsigned long long kdrop = s_drop;
   if (kdrop != ~0ull) {
     long long at = LLONG_MAX;
     for (int h = tid; h < m; h += nt)
@@ -1120,10 +1122,10 @@ __global__ void __launch_bounds__(128) k_bwd_polish(Dev<F> D, BwdDev<F> B) {
         if (v > tol) low = min(low, ~mono_key(v));
       }
     });
-    if (low != ~0ull) atomicMin(&s_key, low);
+    if (low != ~0ull) atomicMin(&s_add, low);
   }
   __syncthreads();
-  const unsigned long long kadd = s_key;
+  const unsigned long long kadd = s_add;
   if (kadd == ~0ull) {
     if (tid == 0) B.pchg[sc] = 0;   // KKT conditions hold
     return;

@@ -1,0 +1,38 @@
+"""Kernels' own sources compiled for the host and run as one CTA on threads
+(host/cuda_runtime.h): schedules of the warps and operands that a GPU run does not
+choose."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+
+def _program(tmp, name):
+    out = os.path.join(str(tmp), name)
+    cc = shutil.which("g++")
+    if cc is None:
+        pytest.skip("needs g++")
+    subprocess.run([cc, "-std=c++20", "-O1", "-ffp-contract=off", "-pthread", "-w", "-I", os.path.join(HERE, "host"), "-I",
+                    os.path.join(ROOT, "paper_2602_15838_gb300", "csrc"), os.path.join(HERE, "host", name + ".cpp"), "-o", out],
+                   check=True, capture_output=True, text=True)
+    return out
+
+
+@pytest.fixture(scope="module")
+def polish(tmp_path_factory):
+    return _program(tmp_path_factory.mktemp("host"), "polish")
+
+
+@pytest.mark.parametrize("what,want", [(0, "0 1 0 0 0 0 1"), (1, "0 0 0 0 0 256 1"), (2, "0 0 0 0 0 0 1")])
+def test_polishing_round_under_every_late_warp(polish, what, want):
+    """One polishing round changes one row, whichever warp comes late after whichever
+    barrier: the row it takes is found in two searches, and a warp that reads the
+    first one's result must not see the second one's."""
+    for warp in range(4):
+        for at in range(8):
+            r = subprocess.run([polish, str(what), str(warp), str(at)], capture_output=True, text=True, timeout=60)
+            assert r.returncode == 0 and r.stdout.strip() == want, (warp, at, r.returncode, r.stdout)
