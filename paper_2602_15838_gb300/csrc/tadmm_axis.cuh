@@ -494,9 +494,13 @@ __device__ void ratio_scan(const AgentCtx<F, NX, NU, DP>& A, bool need, EqpScan<
       den = from_bits(pb, F(0));
       return true;
     };
-    // float32 bounds of the ratio: both operands cut to 24 bits (2^-23 each), one division
+    // float32 bounds of the ratio: both operands cut to 24 bits (2^-23 each), one
+    // division.  A distance that is cut to zero and is not zero has no bounds (NaN:
+    // it stays a candidate and limits no other).
     auto low_of = [&](F num, F den, float& up) -> float {
-      const float r = near_f32(num) / near_f32(den);
+      const float fn = near_f32(num);
+      const bool lost = fn == 0.0f && abs_bits(num) != ord_bits(F(0));
+      const float r = (lost ? __uint_as_float(0x7FC00000u) : fn) / near_f32(den);
       up = r < 1e-30f ? 1e-30f : r * (1.0f + 0x1p-19f);
       return r < 1e-30f ? 0.0f : r * (1.0f - 0x1p-19f);
     };

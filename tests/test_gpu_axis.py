@@ -106,3 +106,11 @@ def test_ratio_test_over_the_lanes(dp, N, T, start):
         assert np.abs(d[k] - g[k]).max(initial=0.0) <= 1e-11 * max(1.0, np.abs(d[k]).max(initial=0.0)), k
     h, ch = _run(b, start=start, mode="graph")
     assert np.array_equal(h["X"], g["X"]) and np.array_equal(ch["eqp"], cg["eqp"])
+
+
+@pytest.mark.parametrize("dp,N,T", [(2, 2, 63), (2, 2, 64), (2, 2, 65), (3, 2, 42), (3, 2, 43)])
+@pytest.mark.parametrize("start", ["turbo", "cold"])
+def test_ratio_test_at_the_edge_of_its_registers(dp, N, T, start):
+    """The ratio test over the lanes keeps 128 inputs of an agent in registers (four per
+    lane) and loads them again beyond: 126 to 130 of them, as above."""
+    test_ratio_test_over_the_lanes(dp, N, T, start)

@@ -36,3 +36,18 @@ def test_polishing_round_under_every_late_warp(polish, what, want):
         for at in range(8):
             r = subprocess.run([polish, str(what), str(warp), str(at)], capture_output=True, text=True, timeout=60)
             assert r.returncode == 0 and r.stdout.strip() == want, (warp, at, r.returncode, r.stdout)
+
+
+@pytest.fixture(scope="module")
+def ratio(tmp_path_factory):
+    return _program(tmp_path_factory.mktemp("host"), "ratio")
+
+
+@pytest.mark.parametrize("what", ["near", "1", "2", "3"])
+def test_ratio_scan_equals_ratio_test(ratio, what):
+    """The ratio test over the lanes takes the blocking input of the test in index
+    order: beside inputs whose distance to a bound float32 cannot tell from 0, and on
+    random steps on either side of what stays in registers (128 inputs)."""
+    r = subprocess.run([ratio, what], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
+    assert int(r.stdout) >= 20
