@@ -229,9 +229,7 @@ static void free_all(tadmm_handle* h) {
   if (!h) return;
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->wexec) cudaGraphExecDestroy(h->wexec);
-  void* gptrs[] = {h->gs_iter, h->gs_active, h->gs_fail, h->gs_rb, h->gs_sb, h->gs_on, h->gs_done, h->gs_blk};
-  for (void* p : gptrs)
-    if (p) cudaFree(p);
+  tadmm::graph_state_free(h);
   void* ptrs0[] = {h->goff, h->gmem, h->gorder};
   for (void* p : ptrs0)
     if (p) cudaFree(p);

@@ -117,6 +117,7 @@ struct tadmm_handle {
        *gs_sb = nullptr, *gs_on = nullptr, *gs_done = nullptr;
   void* gs_blk = nullptr;   // int2 (scenario, first agent) per 32-agent gather block
   int n_gblk = 0;
+  int gs_ready = 0;         // all of these are allocated and the gather table is uploaded
   cudaGraphExec_t wexec = nullptr;
   double w_tol = -1.0;
   int w_iter = -1;
@@ -126,6 +127,35 @@ namespace tadmm {
 
 int set_error(int code, const std::string& msg);
 int cuda_check(cudaError_t e, const char* what);
+
+// Device blocks of the graph mode: all of them or, after a failed allocation, none
+// (the next solve then tries again).
+inline void graph_state_free(tadmm_handle* h) {
+  void** const blocks[] = {&h->gs_iter, &h->gs_active, &h->gs_fail, &h->gs_rb,
+                           &h->gs_sb,   &h->gs_on,     &h->gs_done, &h->gs_blk};
+  for (void** p : blocks) {
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+  }
+  h->gs_ready = 0;
+}
+
+inline int graph_state_alloc(tadmm_handle* h) {
+  graph_state_free(h);
+  const size_t n = (size_t)h->n_scen;
+  const size_t on = (size_t)(h->tot_on > 0 ? h->tot_on : 1), blk = (size_t)(h->n_gblk > 0 ? h->n_gblk : 1);
+  struct { void** p; size_t bytes; } const want[] = {
+      {&h->gs_iter, 4 * n}, {&h->gs_active, 4 * n}, {&h->gs_fail, 4 * n}, {&h->gs_rb, 8 * n},
+      {&h->gs_sb, 8 * n},   {&h->gs_done, 8},       {&h->gs_on, 4 * on},  {&h->gs_blk, 8 * blk}};
+  for (const auto& w : want)
+    if (cudaMalloc(w.p, w.bytes) != cudaSuccess) {
+      cudaGetLastError();
+      *w.p = nullptr;
+      graph_state_free(h);
+      return set_error(TADMM_ENOMEM, "graph-mode state allocation failed");
+    }
+  return TADMM_OK;
+}
 
 template <typename F, int NX, int NU, int DP>
 struct Impl {

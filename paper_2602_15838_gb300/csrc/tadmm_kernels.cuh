@@ -922,18 +922,7 @@ int Impl<F, NX, NU, DP>::solve_plain(tadmm_handle* h, double tol, int max_iter, 
 template <typename F, int NX, int NU, int DP>
 int Impl<F, NX, NU, DP>::solve_graph(tadmm_handle* h, double tol, int max_iter, cudaStream_t st) {
   int rc;
-  if (!h->gs_iter) {
-    const size_t n = (size_t)h->n_scen;
-    if (cudaMalloc(&h->gs_iter, 4 * n) != cudaSuccess || cudaMalloc(&h->gs_active, 4 * n) != cudaSuccess ||
-        cudaMalloc(&h->gs_fail, 4 * n) != cudaSuccess ||
-        cudaMalloc(&h->gs_rb, 8 * n) != cudaSuccess || cudaMalloc(&h->gs_sb, 8 * n) != cudaSuccess ||
-        cudaMalloc(&h->gs_done, 8) != cudaSuccess ||
-        cudaMalloc(&h->gs_on, 4 * (size_t)std::max<int64_t>(h->tot_on, 1)) != cudaSuccess) {
-      cudaGetLastError();
-      return set_error(TADMM_ENOMEM, "graph-mode state allocation failed");
-    }
-  }
-  if (!h->gs_blk) {
+  if (!h->gs_ready) {
     // gather blocks: (scenario, first agent) for every 32 agents of every scenario
     std::vector<int32_t> blk;
     for (int sc = 0; sc < h->n_scen; ++sc)
@@ -942,13 +931,11 @@ int Impl<F, NX, NU, DP>::solve_graph(tadmm_handle* h, double tol, int max_iter, 
         blk.push_back(i0);
       }
     h->n_gblk = (int)(blk.size() / 2);
-    if (cudaMalloc(&h->gs_blk, 4 * std::max<size_t>(blk.size(), 2)) != cudaSuccess) {
-      cudaGetLastError();
-      return set_error(TADMM_ENOMEM, "graph-mode state allocation failed");
-    }
+    if ((rc = graph_state_alloc(h))) return rc;
     if ((rc = cuda_check(cudaMemcpy(h->gs_blk, blk.data(), 4 * blk.size(), cudaMemcpyHostToDevice),
                          "graph-mode gather table")))
       return rc;
+    h->gs_ready = 1;
   }
   GState G{(int32_t*)h->gs_iter, (int32_t*)h->gs_active, (int32_t*)h->gs_fail,
            (unsigned long long*)h->gs_rb, (unsigned long long*)h->gs_sb, (uint32_t*)h->gs_on, (int32_t*)h->gs_done};

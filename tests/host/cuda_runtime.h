@@ -9,6 +9,7 @@
 #include <math.h>
 #include <stddef.h>
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
@@ -170,3 +171,29 @@ template <typename T, typename V>
 T atomicOr(T* p, V v) { return host_atomic(p, [&](T o) { return o | (T)v; }); }
 template <typename T, typename V>
 T atomicAdd(T* p, V v) { return host_atomic(p, [&](T o) { return o + (T)v; }); }
+
+// The runtime calls of the host code under test; a test may let the n-th allocation fail.
+typedef int cudaError_t;
+typedef struct host_stream* cudaStream_t;
+typedef struct host_graph* cudaGraphExec_t;
+enum { cudaSuccess = 0, cudaErrorMemoryAllocation = 2 };
+namespace host_cta {
+inline std::vector<void*> blocks;   // allocated and not freed
+inline int allocations = 0, fail_at = -1;
+}  // namespace host_cta
+inline cudaError_t cudaMalloc(void** p, size_t bytes) {
+  using namespace host_cta;
+  if (allocations++ == fail_at) return cudaErrorMemoryAllocation;   // *p is left as it was
+  *p = malloc(bytes);
+  blocks.push_back(*p);
+  return cudaSuccess;
+}
+inline cudaError_t cudaFree(void* p) {
+  auto& b = host_cta::blocks;
+  const auto at = std::find(b.begin(), b.end(), p);
+  if (at == b.end()) abort();   // freed twice, or never allocated
+  b.erase(at);
+  free(p);
+  return cudaSuccess;
+}
+inline cudaError_t cudaGetLastError() { return cudaSuccess; }

@@ -51,3 +51,11 @@ def test_ratio_scan_equals_ratio_test(ratio, what):
     r = subprocess.run([ratio, what], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
     assert int(r.stdout) >= 20
+
+
+def test_graph_state_after_a_failed_allocation(tmp_path):
+    """Whichever block of the graph mode's state cannot be allocated, the handle keeps
+    none, and the next solve starts over (a later one failing must not leave the first
+    as the mark of a complete state)."""
+    r = subprocess.run([_program(tmp_path, "graph_state")], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and int(r.stdout) == 8, (r.returncode, r.stdout, r.stderr)
