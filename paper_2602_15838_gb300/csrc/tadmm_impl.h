@@ -128,6 +128,31 @@ namespace tadmm {
 int set_error(int code, const std::string& msg);
 int cuda_check(cudaError_t e, const char* what);
 
+// Graph mode: whether everything after an iteration's x-update runs as one CTA per
+// scenario (k_g_tail) and not as grid-wide kernels.  That saves about 5 us of launches
+// an iteration and costs about 3.5 ns per pair-step of the largest scenario, so the
+// line lies near 2000 of them (measured, one scenario, us an iteration against the
+// grid-wide kernels: 14 agents x 20 steps, 1820 pair-steps, -1; 8 x 80, 2240, +4;
+// 20 x 20, 3800, +5; 32 x 20, 9920, +16; 32 x 1280, 635 000, +2195).  Agent-steps count
+// too: each takes its sum.  With more scenarios than one per SM the CTAs fill the GPU
+// and the two are level (256 of 32 agents x 20 steps: -7), unless one of them is longer
+// than an SM's share of all.  k_g_tail holds at most kGroupMax agents, the grid-wide
+// kernels at most 65535 steps.
+constexpr int kTailWork = 2560;
+inline bool tail_per_scenario(const std::vector<ScenMeta>& scen, int sm_count) {
+  int64_t top = 0, total = 0;
+  int nmax = 0, tmax = 0;
+  for (const ScenMeta& m : scen) {
+    const int64_t work = ((int64_t)m.P + m.N) * m.T;
+    top = work > top ? work : top;
+    total += work;
+    nmax = m.N > nmax ? m.N : nmax;
+    tmax = m.T > tmax ? m.T : tmax;
+  }
+  if (nmax > kGroupMax) return false;
+  return top <= kTailWork || top <= total / (sm_count > 0 ? sm_count : 1) || tmax > 65535;
+}
+
 // Device blocks of the graph mode: all of them or, after a failed allocation, none
 // (the next solve then tries again).
 inline void graph_state_free(tadmm_handle* h) {

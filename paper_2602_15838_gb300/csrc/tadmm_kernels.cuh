@@ -328,11 +328,10 @@ __global__ void __launch_bounds__(32) k_g_gather(Dev<F> D, GState G, const int2*
   gather_step<F, NX, NU, DP>(D, s, k1 & 1, k1 % 3, (k1 + 2) % 3, tm1, i, G.on + s.on_off);
 }
 
-// Everything after the x-update of an iteration, one CTA per scenario: for
-// scenarios of at most kGroupMax agents, where four more launches cost an
-// iteration more than the work itself (a 14-agent ring over 300 iterations
-// 18.9 -> 16.7 ms; the rest is the chain of its x-updates).  The last CTA sets the
-// WHILE condition.
+// Everything after the x-update of an iteration, one CTA per scenario: for small
+// scenarios, where four more launches cost an iteration more than the work itself (a
+// 14-agent ring over 300 iterations 18.9 -> 16.7 ms; the rest is the chain of its
+// x-updates).  tail_per_scenario has the rule.  The last CTA sets the WHILE condition.
 constexpr int kTailThreads = 512;
 template <typename F, int NX, int NU, int DP>
 __global__ void __launch_bounds__(kTailThreads) k_g_tail(Dev<F> D, GState G, cudaGraphConditionalHandle cond) {
@@ -987,9 +986,7 @@ int Impl<F, NX, NU, DP>::solve_graph(tadmm_handle* h, double tol, int max_iter, 
         k_g_xupdate<F, NX, NU, DP, false, true><<<gx, 32, 0, h->cap_stream>>>(D, G, h->agent_scen, h->tot_agents, gapw);
       else
         k_g_xupdate<F, NX, NU, DP, false><<<gx, 32, 0, h->cap_stream>>>(D, G, h->agent_scen, h->tot_agents, gapw);
-    int nmax = 0;
-    for (const ScenMeta& m : h->meta_h) nmax = std::max(nmax, m.N);
-    if (nmax <= kGroupMax) {
+    if (tail_per_scenario(h->meta_h, h->sm_count)) {
       k_g_tail<F, NX, NU, DP><<<h->n_scen, kTailThreads, 0, h->cap_stream>>>(D, G, cond);
     } else {
       if (h->tot_pairs > 0) k_g_pair<F, NX, NU, DP><<<gp, 128, 0, h->cap_stream>>>(D, G, h->pair_scen, h->tot_pairs);

@@ -59,3 +59,19 @@ def test_graph_state_after_a_failed_allocation(tmp_path):
     as the mark of a complete state)."""
     r = subprocess.run([_program(tmp_path, "graph_state")], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and int(r.stdout) == 8, (r.returncode, r.stdout, r.stderr)
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    return _program(tmp_path_factory.mktemp("host"), "rules")
+
+
+@pytest.mark.parametrize("scenarios,want", [
+    ([(14, 20, 1)], 1), ([(2, 20, 1)], 1), ([(14, 24, 1)], 1), ([(14, 25, 1)], 0), ([(32, 20, 1)], 0), ([(8, 80, 1)], 0),
+    ([(32, 1280, 1)], 0), ([(32, 20, 64)], 0), ([(32, 20, 256)], 1), ([(4, 20, 300), (32, 2560, 1)], 0), ([(33, 2, 1)], 0),
+    ([(4, 70000, 1)], 1)])
+def test_tail_rule_of_the_graph_mode(rules, scenarios, want):
+    """One CTA per scenario for what comes after the x-update only where the measured
+    times (beside the rule) have it ahead or level: not for long horizons."""
+    r = subprocess.run([rules, "tail", "152"] + [str(v) for s in scenarios for v in s], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and int(r.stdout) == want, r.stdout
