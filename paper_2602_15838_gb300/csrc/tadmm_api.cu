@@ -220,6 +220,7 @@ static void set_structure(tadmm_handle* h, const tadmm_batch* b, int64_t na) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->wexec) cudaGraphExecDestroy(h->wexec);
     h->gexec = h->wexec = nullptr;
+    h->auto_tpc = 0;
   }
   h->di = di;
   h->ax = ax;
@@ -496,7 +497,8 @@ extern "C" int tadmm_create(const tadmm_batch* b, const tadmm_options* opt, tadm
       }
       // groups that run the group path: several scenarios, or one of <= 32 agents
       if (groups[g].size() > 1 || h->N[groups[g][0]] <= 32) h->max_group_pairs = std::max(h->max_group_pairs, gp);
-      gw[g] = double(h->T[groups[g][0]]) * (600.0 + 30.0 * pairs / 32.0);
+      gw[g] = tadmm::group_work(h->T[groups[g][0]], pairs);
+      h->load.add(h->N[groups[g][0]] > tadmm::kGroupMax, gw[g]);
     }
     std::vector<int32_t> gord(groups.size());
     std::iota(gord.begin(), gord.end(), 0);

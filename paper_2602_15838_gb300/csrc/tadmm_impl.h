@@ -5,6 +5,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -24,6 +25,21 @@ struct BwdBufs {
          pchg_cap = 0, set_act_cap = 0, set_W_cap = 0;
 };
 
+namespace tadmm {
+
+// Estimated work of the persistent kernel's groups: those of at most kGroupMax agents
+// ([0]) and the larger scenarios, alone on a CTA ([1]).
+inline double group_work(int T, double pairs) { return T * (600.0 + 30.0 * pairs / 32.0); }
+struct GroupLoad {
+  double sum[2] = {0.0, 0.0}, top[2] = {0.0, 0.0};
+  void add(bool large, double w) {
+    sum[large] += w;
+    top[large] = w > top[large] ? w : top[large];
+  }
+};
+
+}  // namespace tadmm
+
 struct tadmm_handle {
   int prec = 64, nx = 0, nu = 0, dp = 0, n_scen = 0;
   int64_t tot_on = 0;       // words of the graph mode's partner masks
@@ -41,6 +57,7 @@ struct tadmm_handle {
   int32_t* gorder = nullptr;
   int n_groups = 0;
   int max_group_pairs = 0;
+  tadmm::GroupLoad load;        // their estimated work
   int32_t* pairs = nullptr;
   int32_t* deg = nullptr;       // [tot_agents] copies per agent
   int32_t* adj_ptr = nullptr;   // [tot_agents + 1]
@@ -101,6 +118,7 @@ struct tadmm_handle {
 
   // batched mode launch shape and captured graph
   int tpc = 0, cps = 0, variant = 0;
+  int auto_tpc = 0;         // threads per CTA by default_threads (0: not asked for yet)
   int di = 0;               // the shared model is an exact double integrator
   int ax = 0;               // it is, or every agent's own model is axis-separable (tadmm_axis.cuh)
   cudaStream_t cap_stream = nullptr;
@@ -127,6 +145,48 @@ namespace tadmm {
 
 int set_error(int code, const std::string& msg);
 int cuda_check(cudaError_t e, const char* what);
+
+// Threads per CTA of the persistent kernel unless given or tuned; resident: CTAs of 128,
+// 64 and 32 threads that an SM holds of this batch (asked for only with a large scenario).
+//
+// Groups of at most 32 agents: an SM holds eight warps of variant 0 (registers), so as
+// many threads as still let every group run at once (receding horizon, 256 scenarios:
+// 44 ms with 128 threads, 58 with 32; 4096 scenarios, 2223 groups: 361 ms with 32
+// threads, 485 with 64, 734 with 128).  The over-relaxed sweep, all pairs in FP64, takes
+// 128 (512 scenarios, 150 iterations: 173 ms, 224 with 64, 316 with 32).
+//
+// With a larger scenario the CTAs hold its pairs in shared memory too, so an SM holds
+// fewer of the small ones, and the scenario itself may take longer than all the rest.
+// Then the shape of the shortest estimated span: the longest CTA, or all CTAs over the
+// slots, where a CTA of 64 (128) threads takes 0.53 (0.41) of the time of one warp for a
+// group and 0.53 (0.36) for a large scenario, as measured.  20 iterations, ms with 32 /
+// 64 / 128 threads: 1000 small scenarios with one of 64 and one of 200 agents 677 / 346 /
+// 190, with one of 90 agents 233 / 143 / 74; 4000 with one of 64 agents 183 / 139 / 183;
+// 1500 of 40 agents 98 / 89 / 121; 300 of 33 to 48 agents 124 / 71 / 64, 700 of them
+// 131 / 87 / 106.  The estimate takes the fastest of each but the last, where the two
+// spans are within 3 % and it takes 128.
+inline int default_threads(const GroupLoad& load, int n_groups, bool relaxed, int sm_count, const int (&resident)[3]) {
+  const int sm = sm_count > 0 ? sm_count : 1, ng = n_groups > 0 ? n_groups : 1;
+  if (load.sum[1] == 0.0) {
+    const int fit = 8 * 32 * sm / ng;
+    return (fit >= 128 || relaxed) ? 128 : (fit >= 64 ? 64 : 32);
+  }
+  constexpr int kThreads[3] = {128, 64, 32};
+  constexpr double kCost[3][2] = {{0.41, 0.36}, {0.53, 0.53}, {1.0, 1.0}};
+  int best = 128;
+  double span = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    if (resident[k] < 1) continue;
+    const double* c = kCost[k];
+    const double longest = std::max(c[0] * load.top[0], c[1] * load.top[1]);
+    const double s = std::max(longest, (c[0] * load.sum[0] + c[1] * load.sum[1]) / ((double)resident[k] * sm));
+    if (span == 0.0 || s < span) {
+      span = s;
+      best = kThreads[k];
+    }
+  }
+  return best;
+}
 
 // Graph mode: whether everything after an iteration's x-update runs as one CTA per
 // scenario (k_g_tail) and not as grid-wide kernels.  That saves about 5 us of launches

@@ -785,15 +785,13 @@ int Impl<F, NX, NU, DP>::max_ctas_per_sm(int tpc, int variant, const tadmm_handl
 template <typename F, int NX, int NU, int DP>
 int Impl<F, NX, NU, DP>::solve_batched(tadmm_handle* h, double tol, int max_iter, cudaStream_t st) {
   const int var = (h->variant >= 0 && h->variant < kNumVariants) ? h->variant : 0;
-  // Threads per CTA unless given or tuned: registers let an SM hold eight warps of
-  // variant 0, so as many threads as still let every group run at once (receding
-  // horizon, 256 scenarios: 44 ms with 128 threads, 58 with 32; 4096 scenarios,
-  // 2223 groups: 361 ms with 32 threads, 485 with 64, 734 with 128).  The
-  // over-relaxed sweep, all pairs in FP64, takes 128 (512 scenarios, 150
-  // iterations: 173 ms, 224 with 64, 316 with 32).
-  const int fit = 8 * 32 * std::max(h->sm_count, 1) / std::max(h->n_groups, 1);
-  const int want = (fit >= 128 || h->opt.relax_alpha != 1.0) ? 128 : (fit >= 64 ? 64 : 32);
-  int tpc = h->tpc > 0 ? h->tpc : std::min(want, variant_maxt(var));
+  if (h->tpc <= 0 && h->auto_tpc == 0) {
+    const bool large = h->load.sum[1] > 0.0;
+    auto holds = [&](int t) { return large && t <= variant_maxt(var) ? max_ctas_per_sm(t, var, h) : 0; };
+    const int resident[3] = {holds(128), holds(64), holds(32)};
+    h->auto_tpc = default_threads(h->load, h->n_groups, h->opt.relax_alpha != 1.0, h->sm_count, resident);
+  }
+  const int tpc = h->tpc > 0 ? h->tpc : std::min(h->auto_tpc, variant_maxt(var));
   const int occ = max_ctas_per_sm(tpc, var, h);
   if (occ < 1) return set_error(TADMM_EINVAL, "launch shape does not fit the kernel variant");
   int cps = h->cps > 0 ? std::min(h->cps, occ) : occ;

@@ -75,3 +75,24 @@ def test_tail_rule_of_the_graph_mode(rules, scenarios, want):
     times (beside the rule) have it ahead or level: not for long horizons."""
     r = subprocess.run([rules, "tail", "152"] + [str(v) for s in scenarios for v in s], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and int(r.stdout) == want, r.stdout
+
+
+# batches of which every shape was timed (beside the rule): CTAs of 128, 64 and 32 threads
+# that an SM holds, groups (agents, steps, how many), the fastest
+@pytest.mark.parametrize("resident,groups,want", [
+    ((2, 4, 8), [(16, 30, 800), (64, 30, 1), (200, 30, 1)], 128), ((2, 3, 3), [(16, 30, 800), (64, 30, 1)], 128),
+    ((2, 2, 2), [(16, 30, 800), (90, 30, 1)], 128), ((2, 3, 3), [(32, 30, 2200), (64, 30, 1)], 64),
+    ((2, 4, 8), [(32, 30, 2200), (100, 30, 1)], 64), ((2, 4, 7), [(40, 25, 1500)], 64),
+    ((2, 4, 5), [(48, 40, 20), (41, 30, 280)], 128), ((2, 4, 8), [(90, 22, 200)], 128), ((2, 2, 2), [(90, 40, 1)], 128)])
+def test_threads_with_large_scenarios(rules, resident, groups, want):
+    r = subprocess.run([rules, "threads", "152", *map(str, resident), "0"] + [str(v) for g in groups for v in g],
+                       capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and int(r.stdout) == want, r.stdout
+
+
+@pytest.mark.parametrize("groups,relaxed,want", [(190, 0, 128), (304, 0, 128), (305, 0, 64), (608, 0, 64), (609, 0, 32),
+                                                 (2223, 0, 32), (2223, 1, 128)])
+def test_threads_of_small_groups(rules, groups, relaxed, want):
+    r = subprocess.run([rules, "threads", "152", "0", "0", "0", str(relaxed), "20", "30", str(groups)],
+                       capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and int(r.stdout) == want, r.stdout
