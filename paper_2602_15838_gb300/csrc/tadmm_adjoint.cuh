@@ -29,7 +29,7 @@ namespace tadmm {
 struct BwdScen {
   int64_t psi_off;   // per-agent responses [N][T][DP][T][DP]
   int64_t s_off;     // Schur complement [m][m], then the normal matrix [m][m]
-  int64_t v_off;     // vectors [3][m]
+  int64_t v_off;     // vectors [4][m]: the two multipliers, two blocks of scratch
   int32_t m;         // active halfspaces
   int32_t pad;
 };
@@ -123,11 +123,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_count(Dev<F> D, BwdDev<F> B
 // factors of its working set: linear term lin(t, r) on x_t (t = 1..T), initial
 // state x0, inputs of the working set at their bounds (at_bounds) or at zero.
 // Emits every state through outx(t, x) and every input through outu(t, u).
-template <typename F, int NX, int NU, bool DI, class Lin, class OutX, class OutU>
+template <typename F, int NX, int NU, class Lin, class OutX, class OutU>
 __device__ void lq_solve(const Model<F, NX, NU>& Mo, const F* cache, const uint16_t* Wm, int N, int i, int T,
                          Lin lin, const F (&x0)[NX], bool at_bounds, F* kk, OutX outx, OutU outu) {
   using CL = CacheLayout<NX, NU>;
-  constexpr int H = NX / 2;
   auto C = [&](int t, int e) -> F { return cache[((size_t)t * CL::E + e) * N + i]; };
   F pn[NX];
 #pragma unroll
@@ -201,22 +200,14 @@ __device__ void lq_solve(const Model<F, NX, NU>& Mo, const F* cache, const uint1
       }
     }
     F xn[NX];
-    if constexpr (DI) {
 #pragma unroll
-      for (int c = 0; c < H; ++c) {
-        xn[c] = fma(Mo.B[0][0], uv[c], fma(Mo.A[0][H], xv[H + c], xv[c]));
-        xn[H + c] = fma(Mo.B[H][0], uv[c], xv[H + c]);
-      }
-    } else {
+    for (int r = 0; r < NX; ++r) {
+      F acc = 0;
 #pragma unroll
-      for (int r = 0; r < NX; ++r) {
-        F acc = 0;
+      for (int c = 0; c < NX; ++c) acc = fma(Mo.A[r][c], xv[c], acc);
 #pragma unroll
-        for (int c = 0; c < NX; ++c) acc = fma(Mo.A[r][c], xv[c], acc);
-#pragma unroll
-        for (int c = 0; c < NU; ++c) acc = fma(Mo.B[r][c], uv[c], acc);
-        xn[r] = acc;
-      }
+      for (int c = 0; c < NU; ++c) acc = fma(Mo.B[r][c], uv[c], acc);
+      xn[r] = acc;
     }
     outu(t, uv);
     outx(t + 1, xn);
@@ -309,8 +300,10 @@ __device__ __forceinline__ void cta_argmax(F& v, int& i, F* red_v, int* red_i) {
 // entries of a step's column it sums up from consecutive words.
 // With the solves by axis below: 12 polishing rounds and a backward pass over 64
 // scenarios of 16 agents 72.9 -> 38.2 ms, 4 rounds over 9 scenarios of 20 agents
-// (several hundred rows) 489 -> 108 ms.  What is left is mostly warp_backward's
-// chain, m^2 / 2 multiply-adds of 68 cycles.
+// (several hundred rows) 489 -> 108 ms.  What is left in the former (48 to 152 active
+// rows, 1.3 ms of a CTA a round): 45 % the pivoted factor, whose every step waits for
+// its barriers and its sums' loads, and 30 % the substitutions, of which warp_backward
+// is a chain of m^2 / 2 multiply-adds of 68 cycles.
 
 // Rank-revealing Cholesky of the positive semidefinite m x m matrix S (full
 // symmetric storage) by one CTA, with diagonal pivoting: step k takes the
@@ -594,16 +587,16 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_main(Dev<F> D, BwdDev<F> B)
 #pragma unroll
         for (int r = 0; r < NX; ++r) xs[r] = x0(i, r);
         F* kk = B.kks + ((s.agent_off + i) * DP) * (size_t)B.kk_stride;
-        lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T,
-                                [&](int t, int r) { return lin(i, t, r, r < DP); }, xs, at_bounds, kk,
-                                [&](int t, const F (&x)[NX]) {
+        lq_solve<F, NX, NU>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T,
+                            [&](int t, int r) { return lin(i, t, r, r < DP); }, xs, at_bounds, kk,
+                            [&](int t, const F (&x)[NX]) {
 #pragma unroll
-                                  for (int r = 0; r < NX; ++r) outx(i, t, r, x[r]);
-                                },
-                                [&](int t, const F (&u)[NU]) {
+                              for (int r = 0; r < NX; ++r) outx(i, t, r, x[r]);
+                            },
+                            [&](int t, const F (&u)[NU]) {
 #pragma unroll
-                                  for (int c = 0; c < NU; ++c) outu(i, t, c, u[c]);
-                                });
+                              for (int c = 0; c < NU; ++c) outu(i, t, c, u[c]);
+                            });
       }
     }
     __syncthreads();
@@ -681,7 +674,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_main(Dev<F> D, BwdDev<F> B)
           Pt[c][r] = v;
         };
         auto putB = [](int, int, F) {};
-        bad |= factor_stage<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), Pn, mask, rbar, t >= 1 ? qbar : nullptr, 1, put, putB, K, L);
+        bad |= factor_stage<F, NX, NU>(agent_model<F, NX, NU>(D, Mo, s, i), Pn, mask, rbar, t >= 1 ? qbar : nullptr, 1, put, putB, K, L);
 #pragma unroll
         for (int r = 0; r < NU; ++r) {
 #pragma unroll
@@ -747,7 +740,7 @@ __global__ void __launch_bounds__(kBwdThreads) k_bwd_main(Dev<F> D, BwdDev<F> B)
           }
         };
         auto outu = [&](int, const F (&)[NU]) {};
-        lq_solve<F, NX, NU, DI>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, z0, false, kk, outx, outu);
+        lq_solve<F, NX, NU>(agent_model<F, NX, NU>(D, Mo, s, i), cache, Wm, N, i, T, lin, z0, false, kk, outx, outu);
       }
     }
   }

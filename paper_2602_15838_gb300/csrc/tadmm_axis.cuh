@@ -9,7 +9,9 @@
 // general products form those zeros and add them; here they are left out, and
 // every other value is formed by the same operations in the same order, so the
 // results have the same bits.  (The inverse of S keeps the form of the general
-// code, adjugate over determinant, since its rounding is part of that.)
+// code, adjugate over determinant, since its rounding is part of that.  In double-float,
+// where a product by the constant 1 is a rounding of its own in the general products,
+// the results differ by such roundings, at the same distance from float64.)
 //
 // The FP64 pipe bounds these loops: a warp issues one FP64 instruction per about
 // 68 cycles, an SM one per 20, whatever the number of active lanes.  An EQP pass
@@ -55,6 +57,10 @@ __device__ __forceinline__ float near_f32(float v) {
   return fabsf(v) < 0x1p60f ? v : __uint_as_float(0x7FC00000u);
 }
 __device__ __forceinline__ float near_f32(df64 v) { return near_f32(v.hi); }
+
+// Margin of such a test on a sum of a few products: of the sizes' sum (its operands' cuts
+// of 2^-23 and its roundings of 2^-24 stay below 2^-20), and for what a cut to 0 leaves out.
+constexpr float kNearRel = 0x1p-19f, kNearAbs = 1e-17f;
 
 // Part of an agent's data that a lane works on: AX axes from c0 on (all of them,
 // or one when the agents of a round are spread over lanes).  Pointers are those
@@ -383,7 +389,7 @@ __device__ __forceinline__ int axis_pass(const AxisView<F, NX, NU, DP, AX>& V) {
           const float g = (a0 + a1) + (a2 + a3);
           // each product is within 2^-22 of its own, each sum within 2^-23 of the sizes' sum
           const float size = (fabsf(a0) + fabsf(a1)) + (fabsf(a2) + fabsf(a3));
-          const float tol = fmaf(size, 0x1p-19f, 1e-17f);
+          const float tol = fmaf(size, kNearRel, kNearAbs);
           if (!((low ? g : -g) > tol)) found |= (g == g) ? PASS_MULT : (PASS_MULT | PASS_NAN);
         } else {
           const F g = fma(V.k(AC::RB + a), u, fma(g2[a], xv[a], fma(g1[a], xp[a], d[a])));

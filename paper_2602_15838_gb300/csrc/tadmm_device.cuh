@@ -313,13 +313,6 @@ struct AgentCtx {
   }
 };
 
-// Factorization of one stage with inputs in `mask` fixed (Riccati backward
-// recursion of Sec. IV.B restricted to the free inputs):
-//   S = Rbar + B'P B, M = B'P A (fixed rows/cols replaced by identity / zero),
-//   K = -S^{-1} M, P_t = Qbar_t + A'P A + M'K; L receives S^{-1}.
-// DI: A = [[I, dt I], [0, I]], B = [[b1 I], [b2 I]] (double integrator, checked
-// exactly on the host); the products skip the structural zeros and ones but
-// accumulate the remaining terms in the order of the dense loops.
 // Inverse of the symmetric NU x NU matrix S (NU = 2 or 3) by its adjugate;
 // returns 1 unless S is positive definite (Sylvester's criterion: positive
 // leading principal minors).  Si receives the full symmetric inverse.
@@ -366,39 +359,33 @@ __device__ __forceinline__ void neg_sinv(const F (&Si)[NU][NU], const F (&v)[NU]
   }
 }
 
+// Factorization of one stage with inputs in `mask` fixed (Riccati backward
+// recursion of Sec. IV.B restricted to the free inputs):
+//   S = Rbar + B'P B, M = B'P A (fixed rows/cols replaced by identity / zero),
+//   K = -S^{-1} M, P_t = Qbar_t + A'P A + M'K; L receives S^{-1}.
+// Dense products, for models that do not fall apart by axis (tadmm_axis.cuh).
 // P_t entry (r, c), r <= c, is handed to put(r, c, value) as soon as it is
 // formed, and entry (r, a) of P_{t+1} B to putB(r, a, value).
-template <typename F, int NX, int NU, bool DI, class PutP, class PutB>
+template <typename F, int NX, int NU, class PutP, class PutB>
 __device__ __forceinline__ int factor_stage(const Model<F, NX, NU>& Mo, const F (&Pn)[NX][NX],
                                             uint16_t mask, const F* rbar, const F* qdiag, int ks,
                                             PutP&& put, PutB&& putB, F (&K)[NU][NX], F (&L)[NU][NU]) {
-  constexpr int H = NX / 2;
   F PA[NX][NX], PB[NX][NU];
 #pragma unroll
   for (int r = 0; r < NX; ++r) {
-    if constexpr (DI) {
-      const F dt = Mo.A[0][H], b1 = Mo.B[0][0], b2 = Mo.B[H][0];
 #pragma unroll
-      for (int c = 0; c < H; ++c) {
-        PA[r][c] = Pn[r][c];
-        PA[r][H + c] = fma(Pn[r][H + c], F(1), Pn[r][c] * dt);
-        PB[r][c] = fma(Pn[r][H + c], b2, Pn[r][c] * b1);
-      }
-    } else {
+    for (int c = 0; c < NX; ++c) {
+      F acc = 0;
 #pragma unroll
-      for (int c = 0; c < NX; ++c) {
-        F acc = 0;
+      for (int k = 0; k < NX; ++k) acc = fma(Pn[r][k], Mo.A[k][c], acc);
+      PA[r][c] = acc;
+    }
 #pragma unroll
-        for (int k = 0; k < NX; ++k) acc = fma(Pn[r][k], Mo.A[k][c], acc);
-        PA[r][c] = acc;
-      }
+    for (int c = 0; c < NU; ++c) {
+      F acc = 0;
 #pragma unroll
-      for (int c = 0; c < NU; ++c) {
-        F acc = 0;
-#pragma unroll
-        for (int k = 0; k < NX; ++k) acc = fma(Pn[r][k], Mo.B[k][c], acc);
-        PB[r][c] = acc;
-      }
+      for (int k = 0; k < NX; ++k) acc = fma(Pn[r][k], Mo.B[k][c], acc);
+      PB[r][c] = acc;
     }
   }
 #pragma unroll
@@ -413,25 +400,15 @@ __device__ __forceinline__ int factor_stage(const Model<F, NX, NU>& Mo, const F 
     for (int b = 0; b < NU; ++b) {
       const bool fb = (mask >> b) & 0x101;
       F acc = (a == b) ? rbar[a * ks] : F(0);
-      if constexpr (DI) {
-        acc = fma(Mo.B[0][0], PB[a][b], acc);
-        acc = fma(Mo.B[H][0], PB[H + a][b], acc);
-      } else {
 #pragma unroll
-        for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], PB[r][b], acc);
-      }
+      for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], PB[r][b], acc);
       S[a][b] = (fa || fb) ? F(a == b ? 1 : 0) : acc;
     }
 #pragma unroll
     for (int c = 0; c < NX; ++c) {
       F acc = 0;
-      if constexpr (DI) {
-        acc = fma(Mo.B[0][0], PA[a][c], acc);
-        acc = fma(Mo.B[H][0], PA[H + a][c], acc);
-      } else {
 #pragma unroll
-        for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], PA[r][c], acc);
-      }
+      for (int r = 0; r < NX; ++r) acc = fma(Mo.B[r][a], PA[r][c], acc);
       Mm[a][c] = fa ? F(0) : acc;
     }
   }
@@ -453,17 +430,8 @@ __device__ __forceinline__ int factor_stage(const Model<F, NX, NU>& Mo, const F 
 #pragma unroll
       for (int c = r; c < NX; ++c) {
         F acc = (r == c) ? qdiag[r * ks] : F(0);
-        if constexpr (DI) {
-          if (r < H) {
-            acc = acc + PA[r][c];
-          } else {
-            acc = fma(Mo.A[0][H], PA[r - H][c], acc);
-            acc = acc + PA[r][c];
-          }
-        } else {
 #pragma unroll
-          for (int k = 0; k < NX; ++k) acc = fma(Mo.A[k][r], PA[k][c], acc);
-        }
+        for (int k = 0; k < NX; ++k) acc = fma(Mo.A[k][r], PA[k][c], acc);
 #pragma unroll
         for (int k = 0; k < NU; ++k) acc = fma(Mm[k][r], K[k][c], acc);
         put(r, c, acc);
@@ -516,8 +484,8 @@ __device__ void refactor_sweep(const AgentCtx<F, NX, NU, DP>& A, bool own, int d
         if (c != r) A.C(t, CL::P + c * NX + r) = v;
       };
       auto putB = [&](int r, int a, F v) { A.C(t, CL::PB + r * NU + a) = v; };
-      bad_out |= factor_stage<F, NX, NU, false>(*A.M, Pn, mask, A.kc + AC::RB * A.ks,
-                                                t >= 1 ? A.kc + AC::QB * A.ks : nullptr, A.ks, put, putB, K, L);
+      bad_out |= factor_stage<F, NX, NU>(*A.M, Pn, mask, A.kc + AC::RB * A.ks,
+                                         t >= 1 ? A.kc + AC::QB * A.ks : nullptr, A.ks, put, putB, K, L);
 #pragma unroll
       for (int a = 0; a < NU; ++a) {
 #pragma unroll
@@ -1529,7 +1497,7 @@ __device__ __forceinline__ bool pair_pushes(F th, F d, const F (&av)[DP], const 
     g = fmaf(-af, fi - fj, g);
     size = fmaf(fabsf(af), fabsf(fi) + fabsf(fj), size);
   }
-  return !(th == F(0) && g < -fmaf(size, 0x1p-19f, 1e-17f));
+  return !(th == F(0) && g < -fmaf(size, kNearRel, kNearAbs));
 }
 
 // pair_phase of one pair-step, leaving out the pairs that do not push; the others
@@ -2146,6 +2114,7 @@ __device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st,
           if (m >= 0) {
             const uint32_t fij = st.pair[u];
             const int fi = fij & 0xFF, fj = (fij >> 8) & 0xFF;
+            // pair_pushes, written out: called, it costs the sweep 1 to 2 % (355 -> 358..362 ms)
             float g = gs.df[m], size = fabsf(g);
 #pragma unroll
             for (int c = 0; c < DP; ++c) {
@@ -2153,7 +2122,7 @@ __device__ void group_sweep(const Dev<F>& D, GroupSm& gs, GroupStage<F, DP>& st,
               g = fmaf(-af, pi - pj, g);
               size = fmaf(fabsf(af), fabsf(pi) + fabsf(pj), size);
             }
-            want = !(thv[b] == F(0) && g < -fmaf(size, 0x1p-19f, 1e-17f));
+            want = !(thv[b] == F(0) && g < -fmaf(size, kNearRel, kNearAbs));
             if (!want) th_n[qk[b]] = F(0);
           }
           const unsigned ball = __ballot_sync(0xffffffffu, want);
