@@ -713,8 +713,8 @@ def extras(tg, torch, batch, args, peaks):
                                         "2011, Sec. 3.4.3), an extension; parity against the oracle 1e-9")
     from instances import heterogeneous_agents, nearest_neighbour_pairs
     out["heterogeneous_agents"] = timed_solves(tg, torch, heterogeneous_agents(batch, seed=7), args, precision=64)
-    out["heterogeneous_agents"]["note"] = ("per-agent dynamics (seeded velocity damping and mass per agent, dense "
-                                           "products) on the same workload, an extension; parity 1e-9")
+    out["heterogeneous_agents"]["note"] = ("per-agent dynamics (seeded velocity damping and mass per agent, "
+                                           "recursions by axis) on the same workload, an extension; parity 1e-9")
     knn = nearest_neighbour_pairs(batch, 4)
     out["knn_coupling"] = timed_solves(tg, torch, knn, args, precision=64)
     out["knn_coupling"]["note"] = ("listed pairs: each agent coupled to its 4 nearest agents at t = 0 (%d of %d "
